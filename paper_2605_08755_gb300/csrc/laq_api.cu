@@ -571,7 +571,7 @@ laq_status laq_pack(const uint8_t* codes, int64_t K, int64_t N, int bits, void* 
     if (K == 0 || N == 0) return LAQ_OK;
     if (!codes || !packed) return LAQ_ERR_NULL;
     if (!aligned(packed, 16)) return LAQ_ERR_ALIGN;
-    return from_cuda(laq::launch_pack(codes, K, N, bits, static_cast<uint32_t*>(packed),
+    return from_cuda(laq::launch_pack(codes, K, N, bits, static_cast<uint8_t*>(packed),
                                       static_cast<cudaStream_t>(stream)));
 }
 
@@ -584,7 +584,7 @@ laq_status laq_unpack(const void* packed, int64_t K, int64_t N, int bits, uint8_
     if (K == 0 || N == 0) return LAQ_OK;
     if (!codes || !packed) return LAQ_ERR_NULL;
     if (!aligned(packed, 16)) return LAQ_ERR_ALIGN;
-    return from_cuda(laq::launch_unpack(static_cast<const uint32_t*>(packed), K, N, bits, codes,
+    return from_cuda(laq::launch_unpack(static_cast<const uint8_t*>(packed), K, N, bits, codes,
                                         static_cast<cudaStream_t>(stream)));
 }
 

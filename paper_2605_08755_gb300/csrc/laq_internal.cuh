@@ -7,9 +7,9 @@ namespace laq {
 
 cudaError_t launch_quantize_rtn(const uint16_t* W, int64_t K, int64_t N, int bits,
                                 uint8_t* codes, uint16_t* s, uint8_t* z, cudaStream_t stream);
-cudaError_t launch_pack(const uint8_t* codes, int64_t K, int64_t N, int bits, uint32_t* packed,
+cudaError_t launch_pack(const uint8_t* codes, int64_t K, int64_t N, int bits, uint8_t* packed,
                         cudaStream_t stream);
-cudaError_t launch_unpack(const uint32_t* packed, int64_t K, int64_t N, int bits, uint8_t* codes,
+cudaError_t launch_unpack(const uint8_t* packed, int64_t K, int64_t N, int bits, uint8_t* codes,
                           cudaStream_t stream);
 
 // One GEMM launch, fully resolved on the host.
