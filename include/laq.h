@@ -113,6 +113,14 @@ laq_status laq_unpack(const void *packed, int64_t K, int64_t N, int bits, uint8_
                       void *stream);
 
 /*
+ * laq_quantize_pack -- laq_quantize_rtn followed by laq_pack in one kernel, without the codes in
+ * between: the same s, z and packed bytes.  Requirements of both (K % 128 == 0, N % 16 == 0,
+ * W and s 2-byte, packed 16-byte aligned, group 128); empty shapes write nothing.
+ */
+laq_status laq_quantize_pack(const void *W, int64_t K, int64_t N, int bits, int group,
+                             void *packed, void *s, uint8_t *z, void *stream);
+
+/*
  * laq_gemm_wxg128 -- Y[M][N] = X[M][K] * W_hat[K][N], W_hat = s * (q - z) per Eq. (1), the
  * quantized linear layer of the decode step (Sec. 5.2 "Inference", Table 3; App. H).
  *

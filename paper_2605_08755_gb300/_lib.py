@@ -18,7 +18,7 @@ STATUS = {0: "LAQ_OK", 1: "LAQ_ERR_NULL", 2: "LAQ_ERR_BITS", 3: "LAQ_ERR_GROUP",
 
 # Symbols include/laq.h declares.
 EXPORTS = ("laq_status_str", "laq_version", "laq_packed_bytes", "laq_quantize_rtn", "laq_pack",
-           "laq_unpack", "laq_gemm_wxg128", "laq_gemm_plan", "laq_gemm_wxg128_config",
+           "laq_unpack", "laq_quantize_pack", "laq_gemm_wxg128", "laq_gemm_plan", "laq_gemm_wxg128_config",
            "laq_chain_workspace_bytes", "laq_gemm_chain", "laq_gemm_chain_static",
            "laq_gemm_wxg128_prologue",
            "laq_rmsnorm", "laq_qk_norm_rope", "laq_attention_workspace_bytes",
@@ -82,6 +82,7 @@ def lib():
     L.laq_quantize_rtn.argtypes = [P, I64, I64, I, I, P, P, P, P]
     L.laq_pack.argtypes = [P, I64, I64, I, P, P]
     L.laq_unpack.argtypes = [P, I64, I64, I, P, P]
+    L.laq_quantize_pack.argtypes = [P, I64, I64, I, I, P, P, P, P]
     L.laq_gemm_wxg128.argtypes = [P, I64, I64, I64, P, P, P, I, P, P]
     L.laq_gemm_plan.argtypes = [I64, I64, I64, I, I, ctypes.POINTER(GemmConfig)]
     L.laq_gemm_wxg128_config.argtypes = [P, I64, I64, I64, P, P, P, I, P,
@@ -115,7 +116,8 @@ def lib():
     L.laq_pass_workspace_bytes.restype = SZ
     L.laq_pass_prepare.argtypes = [P, P, SZ, P]
     L.laq_pass_run.argtypes = [P, P, P, SZ, P]
-    for name in ("laq_quantize_rtn", "laq_pack", "laq_unpack", "laq_gemm_wxg128",
+    for name in ("laq_quantize_rtn", "laq_pack", "laq_unpack", "laq_quantize_pack",
+                 "laq_gemm_wxg128",
                  "laq_gemm_plan", "laq_gemm_wxg128_config", "laq_gemm_chain",
                  "laq_gemm_chain_static", "laq_rmsnorm", "laq_qk_norm_rope",
                  "laq_gemm_wxg128_prologue",
@@ -176,6 +178,19 @@ def laq_unpack(packed, K, N, bits, stream=None):
     _check(lib().laq_unpack(_ptr(packed), K, N, bits, _ptr(codes), _stream(stream)),
            "laq_unpack")
     return codes
+
+
+def laq_quantize_pack(W, bits, group=128, stream=None):
+    """W [K, N] fp16 (CUDA) -> (packed, s, z): laq_quantize_rtn and laq_pack in one kernel."""
+    import torch
+    K, N = W.shape
+    packed = torch.empty((K * N * bits // 8,), dtype=torch.uint8, device=W.device)
+    s = torch.empty((K // 128, N), dtype=torch.float16, device=W.device)
+    z = torch.empty((K // 128, N), dtype=torch.uint8, device=W.device)
+    W = W.contiguous()
+    _check(lib().laq_quantize_pack(_ptr(W), K, N, bits, group, _ptr(packed), _ptr(s), _ptr(z),
+                                   _stream(stream)), "laq_quantize_pack")
+    return packed, s, z
 
 
 def laq_gemm_wxg128(X, packed, s, z, bits, Y=None, config=None, stream=None):

@@ -557,9 +557,25 @@ laq_status laq_quantize_rtn(const void* W, int64_t K, int64_t N, int bits, int g
     if (K == 0 || N == 0) return LAQ_OK;
     if (!W || !codes || !s || !z) return LAQ_ERR_NULL;
     if (!aligned(W, 2) || !aligned(s, 2)) return LAQ_ERR_ALIGN;
-    return from_cuda(laq::launch_quantize_rtn(static_cast<const uint16_t*>(W), K, N, bits, codes,
-                                              static_cast<uint16_t*>(s), z,
-                                              static_cast<cudaStream_t>(stream)));
+    return from_cuda(laq::launch_quantize(static_cast<const uint16_t*>(W), K, N, bits, codes,
+                                          nullptr, static_cast<uint16_t*>(s), z,
+                                          static_cast<cudaStream_t>(stream)));
+}
+
+laq_status laq_quantize_pack(const void* W, int64_t K, int64_t N, int bits, int group,
+                             void* packed, void* s, uint8_t* z, void* stream) {
+    laq_status st = check_bits(bits);
+    if (st != LAQ_OK) return st;
+    if (group != kGroup) return LAQ_ERR_GROUP;
+    st = check_kn(K, N, true);
+    if (st != LAQ_OK) return st;
+    if (K == 0 || N == 0) return LAQ_OK;
+    if (!W || !packed || !s || !z) return LAQ_ERR_NULL;
+    if (!aligned(W, 2) || !aligned(s, 2) || !aligned(packed, 16)) return LAQ_ERR_ALIGN;
+    return from_cuda(laq::launch_quantize(static_cast<const uint16_t*>(W), K, N, bits, nullptr,
+                                          static_cast<uint8_t*>(packed),
+                                          static_cast<uint16_t*>(s), z,
+                                          static_cast<cudaStream_t>(stream)));
 }
 
 laq_status laq_pack(const uint8_t* codes, int64_t K, int64_t N, int bits, void* packed,

@@ -5,8 +5,9 @@
 
 namespace laq {
 
-cudaError_t launch_quantize_rtn(const uint16_t* W, int64_t K, int64_t N, int bits,
-                                uint8_t* codes, uint16_t* s, uint8_t* z, cudaStream_t stream);
+// Exactly one of codes and packed is given.
+cudaError_t launch_quantize(const uint16_t* W, int64_t K, int64_t N, int bits, uint8_t* codes,
+                            uint8_t* packed, uint16_t* s, uint8_t* z, cudaStream_t stream);
 cudaError_t launch_pack(const uint8_t* codes, int64_t K, int64_t N, int bits, uint8_t* packed,
                         cudaStream_t stream);
 cudaError_t launch_unpack(const uint8_t* packed, int64_t K, int64_t N, int bits, uint8_t* codes,

@@ -12,7 +12,8 @@
 // Bound: HBM for pack and unpack; issue slots (about 10 instructions per weight) and HBM about
 // equally for the quantizer.  The earlier forms divided in fp64 per weight, which GB300's fp64
 // pipe (2 FMAs per clock and SM) held at 1190 us for 2560 x 19456, and gathered (scattered)
-// single code bytes.  Quantize + pack of 2560 x 19456 at 4 bits: 1220 -> 42 us; quantize + pack +
+// single code bytes.  Quantize + pack of 2560 x 19456 at 4 bits: 1220 -> 42 us, in one kernel
+// without the codes between them (laq_quantize_pack) 29 us (126 MB: 4.4 TB/s); quantize + pack +
 // unpack of 12288 x 4096 at 3 bits: 1324 -> 56 us.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -209,15 +210,16 @@ __device__ __forceinline__ __half2 as_half2(uint32_t v) {
     return *reinterpret_cast<const __half2*>(&v);
 }
 
-// Quantize one group of 128 columns.
+// Quantize one group of 128 columns: codes[K][N] (PACK false) or packed records (PACK true).
 // VEC: 8-byte row accesses (N % 4 == 0, W 8-byte and codes 4-byte aligned).
 //
 // All arithmetic is fp32 and still makes exactly the decisions of the rule in laq.h: see
 // quotient() and group_params().
-template <int BITS, bool VEC>
+template <int BITS, bool VEC, bool PACK>
 __global__ void __launch_bounds__(kThreads)
-quantize_kernel(const uint16_t* __restrict__ W, int64_t N, uint8_t* __restrict__ codes,
-                uint16_t* __restrict__ s, uint8_t* __restrict__ z) {
+quantize_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t G, uint8_t* __restrict__ codes,
+                uint8_t* __restrict__ packed, uint16_t* __restrict__ s,
+                uint8_t* __restrict__ z) {
     constexpr int qmax = (1 << BITS) - 1;
     __shared__ __align__(16) uint16_t lo_sm[4][kCols], hi_sm[4][kCols];
     __shared__ __align__(16) float s_sm[kCols], inv_sm[kCols];
@@ -276,6 +278,9 @@ quantize_kernel(const uint16_t* __restrict__ W, int64_t N, uint8_t* __restrict__
     const float sv[4] = {sv4.x, sv4.y, sv4.z, sv4.w}, iv[4] = {iv4.x, iv4.y, iv4.z, iv4.w};
     const int zo[4] = {zv4.x - kMagicBits, zv4.y - kMagicBits, zv4.z - kMagicBits,
                        zv4.w - kMagicBits};
+    const int slot = (lane >> 1) & 1;
+    ColumnWords<BITS> cw;
+    if (PACK) cw.clear();
 #pragma unroll
     for (int i = 0; i < 16; ++i) {  // rows 2i, 2i + 1
         uint32_t q[2][4];
@@ -290,10 +295,19 @@ quantize_kernel(const uint16_t* __restrict__ W, int64_t N, uint8_t* __restrict__
                 q[e][j] = (uint32_t)min(max(__float_as_int(m) + zo[j], 0), qmax);  // then add z
             }
         }
+        if (PACK) {
 #pragma unroll
-        for (int e = 0; e < 2; ++e)
-            store_c4<VEC>(codes + row0 + (2 * i + e) * N,
-                          q[e][0] | q[e][1] << 8 | q[e][2] << 16 | q[e][3] << 24, cols);
+            for (int j = 0; j < 4; ++j) cw.put(j, i, q[0][j] | q[1][j] << 16, slot);
+        } else {
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+                store_c4<VEC>(codes + row0 + (2 * i + e) * N,
+                              q[e][0] | q[e][1] << 8 | q[e][2] << 16 | q[e][3] << 24, cols);
+        }
+    }
+    if constexpr (PACK) {
+        __shared__ Stage<BITS> st;
+        store_records<BITS>(cw, st, n0, N, G, g, packed);
     }
 }
 
@@ -384,19 +398,32 @@ dim3 grid_of(int64_t K, int64_t N) {
     return dim3((unsigned)((N + kCols - 1) / kCols), (unsigned)(K / kGroup));
 }
 
-}  // namespace
-
-cudaError_t launch_quantize_rtn(const uint16_t* W, int64_t K, int64_t N, int bits,
-                                uint8_t* codes, uint16_t* s, uint8_t* z, cudaStream_t stream) {
+template <int BITS>
+void run_quantize(const uint16_t* W, int64_t K, int64_t N, uint8_t* codes, uint8_t* packed,
+                  uint16_t* s, uint8_t* z, cudaStream_t stream) {
+    const int64_t G = K / kGroup;
     const dim3 grid = grid_of(K, N);
     const bool vec = N % 4 == 0 && aligned(W, 8) && aligned(codes, 4);
-    if (bits == 3) {
-        if (vec) quantize_kernel<3, true><<<grid, kThreads, 0, stream>>>(W, N, codes, s, z);
-        else quantize_kernel<3, false><<<grid, kThreads, 0, stream>>>(W, N, codes, s, z);
+    if (packed) {
+        if (vec)
+            quantize_kernel<BITS, true, true><<<grid, kThreads, 0, stream>>>(W, N, G, codes, packed, s, z);
+        else
+            quantize_kernel<BITS, false, true><<<grid, kThreads, 0, stream>>>(W, N, G, codes, packed, s, z);
+    } else if (vec) {
+        quantize_kernel<BITS, true, false><<<grid, kThreads, 0, stream>>>(W, N, G, codes, packed, s, z);
     } else {
-        if (vec) quantize_kernel<4, true><<<grid, kThreads, 0, stream>>>(W, N, codes, s, z);
-        else quantize_kernel<4, false><<<grid, kThreads, 0, stream>>>(W, N, codes, s, z);
+        quantize_kernel<BITS, false, false><<<grid, kThreads, 0, stream>>>(W, N, G, codes, packed, s, z);
     }
+}
+
+}  // namespace
+
+cudaError_t launch_quantize(const uint16_t* W, int64_t K, int64_t N, int bits, uint8_t* codes,
+                            uint8_t* packed, uint16_t* s, uint8_t* z, cudaStream_t stream) {
+    if (bits == 3)
+        run_quantize<3>(W, K, N, codes, packed, s, z, stream);
+    else
+        run_quantize<4>(W, K, N, codes, packed, s, z, stream);
     return cudaGetLastError();
 }
 

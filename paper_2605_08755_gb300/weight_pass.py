@@ -2,9 +2,8 @@
 
 One decode step of a batch-1 (or batch-M) decoder multiplies the current activations by each of
 the 7 projections (q, k, v, o, gate, up, down) of each of the 36 layers (Sec. 5.2, "Inference":
-decoding speed is bounded by streaming these weights).  ``WeightPass`` quantizes synthetic
-weights with ``laq_quantize_rtn``, packs them with ``laq_pack``, and launches the 252
-``laq_gemm_wxg128`` calls in stream order, optionally captured into one CUDA graph.  The
+decoding speed is bounded by streaming these weights).  ``WeightPass`` quantizes and packs synthetic
+weights with ``laq_quantize_pack`` and launches the 252 ``laq_gemm_wxg128`` calls in stream order, optionally captured into one CUDA graph.  The
 activations and outputs are per-projection slices of two flat buffers, so one host-to-device
 copy feeds a whole step and one device-to-host copy returns it (the attention, norms and SiLU
 between the projections are outside this pass).
@@ -19,11 +18,8 @@ class QuantLinear:
 
     def __init__(self, W, bits):
         K, N = W.shape
-        codes, s, z = _lib.laq_quantize_rtn(W, bits)
-        self.packed = _lib.laq_pack(codes, bits)
-        self.s, self.z = s, z
+        self.packed, self.s, self.z = _lib.laq_quantize_pack(W, bits)
         self.K, self.N, self.bits = K, N, bits
-        del codes
 
     def bytes_per_call(self, M):
         """Algorithmic HBM bytes of one call: packed codes + s (2 B) + z (1 B) per (group,

@@ -78,6 +78,26 @@ def test_quantizer_at_edges(bits, K, N, offset):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("bits", [3, 4])
+@pytest.mark.parametrize("K,N,offset", [(128, 16, 0), (256, 112, 0), (384, 4096, 0), (256, 144, 1),
+                                        (128, 272, 2), (256, 1040, 4)])
+def test_fused_quantize_pack_at_edges(bits, K, N, offset):
+    """The packed records, scales and zeros are those of the quantizer and packer of the oracle."""
+    import torch
+    from paper_2605_08755_gb300 import _lib, build
+    build.build()
+    W = _matrix(K, N, seed=K + N + offset)
+    buf = torch.zeros(K * N + offset, dtype=torch.float16, device="cuda")
+    buf[offset:] = torch.from_numpy(W).cuda().flatten()
+    packed, s, z = _lib.laq_quantize_pack(buf[offset:].view(K, N), bits)
+    torch.cuda.synchronize()
+    rc, rs, rz = co.quantize_rtn(W, bits)
+    assert np.array_equal(packed.cpu().numpy().view(np.uint32), co.pack(rc, bits))
+    assert np.array_equal(s.cpu().numpy().view(np.uint16), rs.view(np.uint16))
+    assert np.array_equal(z.cpu().numpy(), rz)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("bits", [3, 4])
 @pytest.mark.parametrize("K,N,offset", [(128, 16, 0), (256, 112, 0), (128, 144, 1), (384, 272, 2),
                                         (256, 1040, 4)])
 def test_pack_and_unpack_at_edges(bits, K, N, offset):
