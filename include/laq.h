@@ -367,7 +367,7 @@ laq_status laq_gemm_wxg128_prologue(const void *X, int64_t M, int64_t K, int64_t
  * LAQ_ERR_NULL, nothing launched); values read from device memory (positions, lengths,
  * tokens) are clamped in the kernels as stated and never index outside the given buffers.
  * Each kernel may start while its predecessor on the stream finishes (programmatic dependent
- * launch) and waits for it before touching memory.
+ * launch) and waits for it before reading or writing anything its results depend on.
  * ====================================================================================== */
 
 /*
@@ -397,17 +397,20 @@ laq_status laq_qk_norm_rope(const void *qkv, const void *q_norm_w, const void *k
                             float theta, float eps, void *q_out, void *k_cache, void *v_cache,
                             int64_t L_max, void *stream);
 
-/* Bytes of workspace laq_attention_decode needs (fp32 partials of 64-token chunks); 0 for
- * invalid sizes. */
+/* Bytes of workspace laq_attention_decode needs (fp32 partials, room for one per 64 tokens); 0
+ * for invalid sizes. */
 size_t laq_attention_workspace_bytes(int64_t M, int32_t Hq, int64_t L_max);
 
 /*
  * Grouped-query attention of each row's new token over its cache (decode):
  *   out[m][h] = sum_{t < n} softmax_t(scale * q[m][h] . K[m][g][t]) V[m][g][t],  g = h / (Hq/Hkv),
  * n = len[m] (device) clamped to [0, L_max]; a row with n = 0 gets zeros.  q, out [M][Hq][D],
- * caches [M][Hkv][L_max][D], D = 128, Hq / Hkv <= 8.  Two launches: 64-token chunk partials
- * (max, sum of exponentials, weighted V sum) into `workspace`, then their combination in chunk
- * order (deterministic).  workspace_bytes >= laq_attention_workspace_bytes(M, Hq, L_max)
+ * caches [M][Hkv][L_max][D], D = 128, Hq / Hkv <= 8.  One launch (a cluster of CTAs per row and
+ * kv head), or, for long caches of few rows and kv heads, partials in `workspace` (max, sum of
+ * exponentials, weighted V sum) and a second launch that combines them; summation orders are
+ * fixed (deterministic).  Before the preceding kernel has finished, the kernel only reads len and
+ * prefetches cache rows into L2; everything its results depend on is read afterwards.
+ * workspace_bytes >= laq_attention_workspace_bytes(M, Hq, L_max)
  * (LAQ_ERR_WORKSPACE otherwise; 4-byte aligned).  Both caches 16-byte aligned.
  */
 laq_status laq_attention_decode(const void *q, const void *k_cache, const void *v_cache,
@@ -420,11 +423,11 @@ laq_status laq_attention_decode(const void *q, const void *k_cache, const void *
 size_t laq_attention_qkv_workspace_bytes(int64_t M, int32_t Hq, int32_t Hkv, int64_t L_max);
 
 /*
- * laq_qk_norm_rope followed by laq_attention_decode with len[m] = pos[m] + 1, in two launches
- * instead of three (same inputs, outputs and results): each attention CTA (64-token chunk, kv
- * head, row) normalises and rotates its q heads itself, and the CTA whose chunk holds pos[m]
+ * laq_qk_norm_rope followed by laq_attention_decode with len[m] = pos[m] + 1, without the launch
+ * between them (same inputs, outputs and results): each attention CTA (part of the tokens, kv
+ * head, row) normalises and rotates its q heads itself, and the warp whose tokens include pos[m]
  * computes the new k and v, stores them in the caches and uses them in place of the cached
- * row; the chunk partials are then combined in chunk order.  Workspace 16-byte aligned and
+ * row.  Workspace 16-byte aligned and
  * >= laq_attention_qkv_workspace_bytes (LAQ_ERR_WORKSPACE otherwise).
  */
 laq_status laq_attention_qkv(const void *qkv, const void *q_norm_w, const void *k_norm_w,

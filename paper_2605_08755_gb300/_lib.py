@@ -397,7 +397,7 @@ def attention_qkv_workspace(M, Hq, Hkv, L_max, device):
 
 def laq_attention_qkv(qkv, q_norm_w, k_norm_w, pos, Hq, Hkv, theta, eps, k_cache, v_cache,
                       scale, workspace, out=None, stream=None):
-    """laq_qk_norm_rope + laq_attention_decode (len = pos + 1) in two launches: out [M, Hq, 128];
+    """laq_qk_norm_rope + laq_attention_decode (len = pos + 1) in one call: out [M, Hq, 128];
     appends k, v at pos[m] to the caches [M, Hkv, L_max, 128]."""
     import torch
     M = qkv.shape[0]

@@ -1,28 +1,34 @@
 // laq_decode.cu -- the decoder operations around the quantized projections of one decode step
 // of a Qwen3-style model (the models whose decoding speed Sec. 5.2 reports): RMSNorm with the
 // residual add, per-head q/k RMSNorm with rotary position embedding and the KV-cache append,
-// grouped-query attention of the new token over its cache (flash-decoding: per-chunk partial
-// softmax, then a combine in chunk order), SiLU(gate) * up, the embedding gather and the greedy
+// grouped-query attention of the new token over its cache (the tokens split over the warps of a
+// cluster of CTAs, combined in a fixed order), SiLU(gate) * up, the embedding gather and the greedy
 // argmax.  The paper defines none of them; they follow the standard decoder definitions, with
 // fp32 arithmetic and one fp16 rounding per stored tensor.
 //
 // Every kernel lets its successor launch at once (griddepcontrol.launch_dependents) and waits
-// for its predecessor (griddepcontrol.wait) before touching memory, so inside a CUDA graph of
+// for its predecessor (griddepcontrol.wait) before reading or writing what its results depend on
+// (attention prefetches cache rows into L2 before), so inside a CUDA graph of
 // programmatically dependent launches each one's launch and set-up overlap the previous one.
+#include <cooperative_groups.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "laq.h"
 #include "laq_device.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace laq {
 namespace {
 
 constexpr int kHeadDim = 128;    // D: the only head size the attention kernels are built for
 constexpr int kMaxGroup = 8;     // most q heads per kv head
-constexpr int kChunk = 64;       // tokens per attention partial
-constexpr int kPartial = kHeadDim + 2;  // floats per (row, q head, chunk): acc[D], max, sum
+constexpr int kChunk = 64;       // tokens per partial that the workspace has room for
+constexpr int kPartial = kHeadDim + 2;  // floats per partial: acc[D], max, sum
 
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
@@ -200,295 +206,420 @@ __global__ void __launch_bounds__(128) qk_norm_rope_kernel(
     }
 }
 
-// The attention of one 64-token chunk whose K and V rows are staged in shared memory, for the
-// G q heads of a kv head (qs: [G][D] fp32, already scaled), written to the partial slots
-// part[j * nchunk * kPartial] (acc[D], max, sum) of head j.  Scores: a half-warp per token
-// (lane l & 15 holds q and k elements 8 (l & 15) .. +7; q in registers); probabilities stored
-// token-major (sc [kChunk][kMaxGroup]) so that one broadcast load gives every head's value of a
-// token; weighted V sum: warp w takes tokens w, w + 4, ..., lane l dimensions 4l .. 4l+3, then
-// the four warps' sums are added in warp order (red aliases the K rows, no longer needed).
-// Every thread of the CTA must call it.
-__device__ __forceinline__ void chunk_core(const __half (*ks)[kHeadDim],
-                                           const __half (*vs)[kHeadDim], const float* qs,
-                                           float* sc, float* mxs, float* sms, int nt, int G,
-                                           float* part, int nchunk) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, hl = lane & 15;
-    float qr[kMaxGroup][8];
-#pragma unroll
-    for (int j = 0; j < kMaxGroup; ++j)
-#pragma unroll
-        for (int e = 0; e < 8; ++e) qr[j][e] = j < G ? qs[j * kHeadDim + 8 * hl + e] : 0.f;
-    for (int base = 0; base < nt; base += 8) {
-        const int tt = base + 2 * warp + (lane >> 4);
-        float kv[8];
-        if (tt < nt) {
-            unpack8(*reinterpret_cast<const uint4*>(&ks[tt][8 * hl]), kv);
-        } else {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) kv[e] = 0.f;
-        }
-#pragma unroll
-        for (int j = 0; j < kMaxGroup; ++j) {
-            if (j >= G) break;  // uniform
-            float s = 0.f;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) s = fmaf(qr[j][e], kv[e], s);
-#pragma unroll
-            for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (hl == 0 && tt < nt) sc[tt * kMaxGroup + j] = s;
-        }
-    }
-    __syncthreads();
-    for (int j = warp; j < G; j += 4) {
-        const float a = lane < nt ? sc[lane * kMaxGroup + j] : -INFINITY;
-        const float b = lane + 32 < nt ? sc[(lane + 32) * kMaxGroup + j] : -INFINITY;
-        float v = fmaxf(a, b);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-        const float pa = lane < nt ? expf(a - v) : 0.f;
-        const float pb = lane + 32 < nt ? expf(b - v) : 0.f;
-        if (lane < nt) sc[lane * kMaxGroup + j] = pa;
-        if (lane + 32 < nt) sc[(lane + 32) * kMaxGroup + j] = pb;
-        const float s = warp_sum(pa + pb);
-        if (lane == 0) {
-            mxs[j] = v;
-            sms[j] = s;
-        }
-    }
-    __syncthreads();
-    float acc[kMaxGroup][4];
-#pragma unroll
-    for (int j = 0; j < kMaxGroup; ++j)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
-    for (int tt = warp; tt < nt; tt += 4) {
-        float vv[4];
-        load4(&vs[tt][4 * lane], vv);
-        const float4 p0 = *reinterpret_cast<const float4*>(sc + tt * kMaxGroup);
-        const float4 p1 = *reinterpret_cast<const float4*>(sc + tt * kMaxGroup + 4);
-        const float pj[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
-#pragma unroll
-        for (int j = 0; j < kMaxGroup; ++j)
-            if (j < G)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) acc[j][e] = fmaf(pj[j], vv[e], acc[j][e]);
-    }
-    float* red = reinterpret_cast<float*>(const_cast<__half*>(&ks[0][0]));  // [4][G][D]
-#pragma unroll
-    for (int j = 0; j < kMaxGroup; ++j)
-        if (j < G)
-            *reinterpret_cast<float4*>(red + ((size_t)warp * G + j) * kHeadDim + 4 * lane) =
-                make_float4(acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
-    __syncthreads();
-    const int d = threadIdx.x;
-    for (int j = 0; j < G; ++j) {
-        float a = 0.f;
-#pragma unroll
-        for (int w = 0; w < 4; ++w) a += red[((size_t)w * G + j) * kHeadDim + d];
-        float* pp = part + (size_t)j * nchunk * kPartial;
-        pp[d] = a;
-        if (d == 0) {
-            pp[kHeadDim] = mxs[j];
-            pp[kHeadDim + 1] = sms[j];
-        }
-    }
+// ---- grouped-query attention of one decode step ----
+// One cluster of C CTAs works on one (row, kv head): the row's n cached tokens are cut into steps
+// of 16, dealt round robin to the cluster's warps, so the split follows the actual length.  A
+// warp streams its steps' K and V rows (2 x 4 KB) through a private cp.async ring and keeps the
+// online softmax of its own tokens for the G = Hq / Hkv q heads at once, on the tensor cores
+// (m16n8k16, fp16 operands, fp32 accumulation):
+//   scores^T = K q^T: A the 16 tokens' K rows straight from ldmatrix, B the q heads (fp16, as
+//     stored; the products are exact);
+//   out^T += V^T P^T: A from ldmatrix.trans, B the probabilities after a movmatrix transpose.
+//     They stay at fp32 precision: P = hi + lo with both halves fp16.  For G <= 4 the MMA's 8
+//     columns are 4 heads' hi and 4 heads' lo (q's B columns 4-7 repeat heads 0-3, so the lanes
+//     that would idle hold the same probabilities and contribute their low halves); WIDE
+//     (G = 5..8) issues one MMA for each half.  hi + lo is P to ~2^-22; p is scaled by 2^15 (it
+//     cancels against the sum of p), so that its small values stay above fp16's range.
+// The warps' results meet in shared memory, the CTAs' through distributed shared memory: CTA r of
+// the cluster combines the head dimensions [128 r / C, 128 (r + 1) / C) in rank order and stores
+// fp16, so a call needs one launch and no scratch.  (Partials in a workspace and a combine kernel,
+// fp32 FMAs and a 4-shuffle score: 13.3 us a call for one row of 2048 tokens, 138 us for 16 rows of
+// 2048 .. 8192; this form 6.7 and 59 us, 5.7 TB/s.)  Where the clusters of all (row, kv head)
+// pairs leave most SMs idle and the rows may be long, S clusters share a pair, write fp32 partials
+// (acc[D], max, sum) to the workspace, and attn_combine_kernel adds them in order.
+// Bound: HBM for long batches; for one short row the latency of a dependent launch (4.6 us at 256
+// tokens) plus about 1 us per step of a warp.  So the ring is one step deep and the CTA has 8
+// warps: at the same shared memory 4 warps with two steps measured 1301 us for a decode step at
+// 2048 tokens against 1261; 16 warps an SM overlap each other's copies and arithmetic.  K and V
+// loaded straight into MMA operand registers (no ring) was slower (249 us against 167 for 24
+// calls), and 131 KB rings keep a CTA from sharing an SM with the kernels before and after it.
+// Swizzle: 16-byte chunk j of a 256-byte row sits at j ^ (row & 7), so the 8 rows of an ldmatrix
+// phase hit different banks.
+constexpr int kStep = 16;                   // tokens per warp step
+constexpr int kAttnWarps = 8;
+constexpr int kAttnStages = 1;              // ring depth, steps (see the comment above)
+constexpr int kStepBytes = 2 * kStep * kHeadDim * 2;  // K and V rows of a step
+constexpr int kMaxCluster = 16;
+constexpr int kRedRow = kHeadDim + 4;       // floats per row of red (lanes of a store: 32 banks)
+
+struct AttnSmem {
+    uint8_t ring[kAttnWarps][kAttnStages][kStepBytes];  // later red[warp][G][kRedRow] fp32
+    uint8_t q[kMaxGroup * kHeadDim * 2];                // fp16 q heads, swizzled rows
+    float recv[kMaxGroup * kHeadDim];                   // [C][G][128 / C] partials of this slice
+    float2 ml[kMaxCluster][kMaxGroup];                  // (max, sum) of every CTA of the cluster
+    float2 wml[kAttnWarps][kMaxGroup];                  // (max, sum) of every warp
+};
+
+struct AttnParams {
+    const __half* q;        // [M][Hq][D], or qkv [M][Hq + 2 Hkv][D] (fused form)
+    const __half* qw;       // fused: q and k norm weights
+    const __half* kw;
+    const int32_t* len;     // cached tokens per row; fused: positions (tokens - 1)
+    __half* k_cache;
+    __half* v_cache;
+    __half* out;
+    float* part;            // S > 1: [M][Hq][S][kPartial]
+    int64_t L_max;
+    int Hq, Hkv, C, S;
+    float log2_theta, eps, scale;
+};
+
+__device__ __forceinline__ void cp_async16_zfill(uint32_t dst, const void* src, bool ok) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src),
+                 "r"(ok ? 16 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void ldsm4(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+__device__ __forceinline__ void ldsm4t(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+// transpose of an 8 x 8 matrix of 16-bit values spread over the warp (two per lane)
+__device__ __forceinline__ uint32_t movmatrix(uint32_t v) {
+    uint32_t r;
+    asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;\n" : "=r"(r) : "r"(v));
+    return r;
+}
+// byte offset of 16-byte chunk j of row r
+__device__ __forceinline__ int swz(int r, int j) { return r * 256 + ((j ^ (r & 7)) << 4); }
+
+__device__ __forceinline__ float exp2_diff(float a, float b) {  // 2^(a - b); a = -inf: 0
+    return a == -INFINITY ? 0.f : exp2f(a - b);
 }
 
-// ---- attention: per-chunk partials ----
-// CTA (chunk c, kv head g, row m) over tokens [64c, 64c + 64) of the row's cached tokens, for
-// the G = Hq / Hkv q heads of g at once (their K and V rows are read once): the chunk's K and V
-// rows (2 x 16 KB) are copied to shared memory with every copy in flight at once, then scores
-// s = scale * q . k, the chunk max, p = exp(s - max), sum p and acc = sum p v, written as
-// partial [m][h][c] = (acc[D], max, sum).  Chunks at or past the row's length write nothing.
-__global__ void __launch_bounds__(128) attn_partial_kernel(
-    const __half* __restrict__ q, const __half* __restrict__ k_cache,
-    const __half* __restrict__ v_cache, const int32_t* __restrict__ len, int Hq, int Hkv,
-    int64_t L_max, float scale, float* part, int nchunk) {
+template <bool FUSED, bool WIDE>
+__global__ void __launch_bounds__(kAttnWarps * 32) attn_kernel(const AttnParams p) {
     pdl_launch_dependents();
-    pdl_wait();
-    __shared__ __align__(16) __half ks[kChunk][kHeadDim];
-    __shared__ __align__(16) __half vs[kChunk][kHeadDim];
-    __shared__ __align__(16) float qs[kMaxGroup * kHeadDim];
-    __shared__ __align__(16) float sc[kChunk * kMaxGroup];
-    __shared__ float mx[kMaxGroup], sm[kMaxGroup];
-    const int c = blockIdx.x, g = blockIdx.y, m = blockIdx.z;
-    const int G = Hq / Hkv;
-    const int L = (int)min((int64_t)max(len[m], 0), L_max);  // cached tokens of row m
-    const int t0 = c * kChunk;
-    if (t0 >= L) return;
-    const int nt = min(kChunk, L - t0);
-    const size_t kv0 = ((size_t)m * Hkv + g) * L_max + t0;  // row of token t0
+    if (p.C > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");
+    extern __shared__ __align__(128) uint8_t attn_smem[];
+    AttnSmem& sm = *reinterpret_cast<AttnSmem*>(attn_smem);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, c = lane & 3, r = lane >> 2;
+    const int g = blockIdx.y, m = blockIdx.z, G = p.Hq / p.Hkv;
+    const int C = p.C, rank = blockIdx.x % C;
+    const int wi = blockIdx.x * kAttnWarps + warp, nw = gridDim.x * kAttnWarps;
+    const size_t kv0 = ((size_t)m * p.Hkv + g) * p.L_max * kHeadDim;
+    // While the preceding kernel finishes: ask L2 for the K and V rows of the warp's first steps
+    // and compute the rotation angles, both by the position as it is now.  A prefetch returns no
+    // data (whatever the preceding kernel still writes is seen by the loads below), and the
+    // position is read again after the wait and the angles redone if it has changed.
+    const int32_t pos_hint = *(const volatile int32_t*)(p.len + m);
+    float cs[4], sn[4];
     {
-        const uint32_t kss = (uint32_t)__cvta_generic_to_shared(&ks[0][0]);
-        const uint32_t vss = (uint32_t)__cvta_generic_to_shared(&vs[0][0]);
-        for (int u = threadIdx.x; u < nt * (kHeadDim / 8); u += blockDim.x) {  // 16-byte pieces
-            cp_async16(kss + 16 * u, k_cache + kv0 * kHeadDim + 8 * u);
-            cp_async16(vss + 16 * u, v_cache + kv0 * kHeadDim + 8 * u);
-        }
-        cp_async_commit();
-    }
-    for (int i = threadIdx.x; i < G * kHeadDim; i += blockDim.x)
-        qs[i] = scale * __half2float(q[((size_t)m * Hq + g * G) * kHeadDim + i]);
-    asm volatile("cp.async.wait_all;\n" ::: "memory");
-    __syncthreads();
-    chunk_core(ks, vs, qs, sc, mx, sm, nt, G,
-               part + (((size_t)m * Hq + g * G) * nchunk + c) * kPartial, nchunk);
-}
-
-// ---- attention: combine the chunk partials ----
-// out[m][h][d] = sum_c e^(max_c - M) acc_c[d] / sum_c e^(max_c - M) sum_c, M = max_c max_c.
-// 512 threads: each chunk's (max, sum) is read once, by one thread, into shared memory; the
-// four 128-thread groups q take the chunks c = q mod 4 (8 independent loads in flight per
-// thread) and their sums are added in group order; the denominator by warp 0.  Fixed orders:
-// the result is deterministic.
-constexpr int kCombineMax = 2048;  // chunks held in shared memory per pass
-constexpr int kCombineThreads = 512;
-__global__ void __launch_bounds__(kCombineThreads) attn_combine_kernel(
-    const float* __restrict__ part, const int32_t* __restrict__ len, int len_is_pos, int Hq,
-    int nchunk, __half* out) {
-    pdl_launch_dependents();
-    pdl_wait();
-    __shared__ float fs[kCombineMax], ss[kCombineMax];
-    __shared__ float red[kCombineThreads / 32];
-    __shared__ float nums[4][kHeadDim];
-    __shared__ float den_s;
-    const int h = blockIdx.x, m = blockIdx.y, tid = threadIdx.x;
-    const int d = tid & (kHeadDim - 1), q = tid >> 7;
-    const int64_t n = (int64_t)len[m] + (len_is_pos ? 1 : 0);
-    const int nc = (int)((min(max(n, (int64_t)0), (int64_t)nchunk * kChunk) + kChunk - 1) /
-                         kChunk);
-    __half* o = out + ((size_t)m * Hq + h) * kHeadDim;
-    if (nc == 0) {  // no cached token: zeros
-        if (q == 0) o[d] = __float2half_rn(0.f);
-        return;
-    }
-    const float* pp = part + ((size_t)m * Hq + h) * nchunk * kPartial;
-    // M = max over all chunks (order-independent); the first pass's (max, sum) stay in smem
-    const int n0 = min(kCombineMax, nc);
-    float lm = -INFINITY;
-    for (int cc = tid; cc < nc; cc += kCombineThreads) {
-        const float mc = pp[(size_t)cc * kPartial + kHeadDim];
-        lm = fmaxf(lm, mc);
-        if (cc < n0) {
-            fs[cc] = mc;
-            ss[cc] = pp[(size_t)cc * kPartial + kHeadDim + 1];
-        }
-    }
+        const int64_t nh = min((int64_t)pos_hint + (FUSED ? 1 : 0), p.L_max);
 #pragma unroll
-    for (int w = 16; w > 0; w >>= 1) lm = fmaxf(lm, __shfl_xor_sync(0xffffffffu, lm, w));
-    if ((tid & 31) == 0) red[tid >> 5] = lm;
-    __syncthreads();
-    float M = red[0];
-#pragma unroll
-    for (int k = 1; k < kCombineThreads / 32; ++k) M = fmaxf(M, red[k]);
-    float num = 0.f, dl = 0.f;  // dl: warp 0's share of the denominator
-    for (int c0 = 0; c0 < nc; c0 += kCombineMax) {
-        const int cnt = min(kCombineMax, nc - c0);
-        if (c0 > 0) {
-            __syncthreads();  // the previous pass is done with fs / ss
-            for (int cc = tid; cc < cnt; cc += kCombineThreads) {
-                fs[cc] = pp[(size_t)(c0 + cc) * kPartial + kHeadDim];
-                ss[cc] = pp[(size_t)(c0 + cc) * kPartial + kHeadDim + 1];
+        for (int i = 0; i < kAttnStages; ++i) {
+            const int64_t t = (int64_t)(wi + i * nw) * kStep + (lane >> 1);
+            if (t < nh) {  // half a row of 128 bytes per lane
+                const size_t off = kv0 + (size_t)t * kHeadDim + 64 * (lane & 1);
+                asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p.k_cache + off));
+                asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p.v_cache + off));
             }
         }
-        __syncthreads();
-        for (int cc = tid; cc < cnt; cc += kCombineThreads) fs[cc] = expf(fs[cc] - M);
-        __syncthreads();
-        if (tid < 32)
-            for (int cc = tid; cc < cnt; cc += 32) dl = fmaf(fs[cc], ss[cc], dl);
-        int cc = q;
-        for (; cc + 28 < cnt; cc += 32) {  // 8 chunks of this group per round
-            float a[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) a[u] = pp[(size_t)(c0 + cc + 4 * u) * kPartial + d];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) num = fmaf(fs[cc + 4 * u], a[u], num);
-        }
-        for (; cc < cnt; cc += 4) num = fmaf(fs[cc], pp[(size_t)(c0 + cc) * kPartial + d], num);
+        if (FUSED) rope_angles(lane, pos_hint, p.log2_theta, cs, sn);
     }
-    if (tid < 32) {
-        dl = warp_sum(dl);
-        if (tid == 0) den_s = dl;
-    }
-    nums[q][d] = num;
-    __syncthreads();
-    if (q == 0)
-        o[d] = __float2half_rn((nums[0][d] + nums[1][d] + nums[2][d] + nums[3][d]) / den_s);
-}
-
-// ---- attention partials with the q/k norm, rotation and cache append folded in ----
-// CTA (chunk c, kv head g, row m), n = clamp(pos[m] + 1, 0, L_max) tokens: the CTA normalises
-// and rotates its G q heads (warp j: head g G + j), stages its chunk's cached K and V, and if
-// the chunk holds position pos[m] (< L_max) computes the new k (norm, rotation) and v, stores
-// them in the caches and uses them in place of the staged row.  Then the chunk partial as in
-// attn_partial_kernel, combined by attn_combine_kernel with len = n.
-__global__ void __launch_bounds__(128) attn_qkv_kernel(
-    const __half* __restrict__ qkv, const __half* __restrict__ qw, const __half* __restrict__ kw,
-    const int32_t* __restrict__ pos, int Hq, int Hkv, float log2_theta, float eps,
-    __half* k_cache, __half* v_cache, int64_t L_max, float scale, float* part, int nchunk) {
-    pdl_launch_dependents();
     pdl_wait();
-    __shared__ __align__(16) __half ks[kChunk][kHeadDim];
-    __shared__ __align__(16) __half vs[kChunk][kHeadDim];
-    __shared__ __align__(16) float qs[kMaxGroup * kHeadDim];
-    __shared__ __align__(16) float sc[kChunk * kMaxGroup];
-    __shared__ float mx[kMaxGroup], sm[kMaxGroup];
-    const int c = blockIdx.x, g = blockIdx.y, m = blockIdx.z;
-    const int G = Hq / Hkv, nh = Hq + 2 * Hkv;
-    const int64_t p = pos[m];
-    const int n = (int)min(max(p + 1, (int64_t)0), L_max);  // tokens attended
-    const int t0 = c * kChunk;
-    if (t0 >= n) return;
-    const int nt = min(kChunk, n - t0);
-    const bool holds_new = p >= t0 && p < t0 + nt;  // (then p < L_max)
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const size_t kv0 = ((size_t)m * Hkv + g) * L_max + t0;
-    {
-        const uint32_t kss = (uint32_t)__cvta_generic_to_shared(&ks[0][0]);
-        const uint32_t vss = (uint32_t)__cvta_generic_to_shared(&vs[0][0]);
-        for (int u = threadIdx.x; u < nt * (kHeadDim / 8); u += blockDim.x) {
-            cp_async16(kss + 16 * u, k_cache + kv0 * kHeadDim + 8 * u);
-            cp_async16(vss + 16 * u, v_cache + kv0 * kHeadDim + 8 * u);
+
+    const int64_t pos = *(const volatile int32_t*)(p.len + m);  // fused: the new token's position
+    constexpr int kPerWarp = kMaxGroup / kAttnWarps;  // q heads a warp prepares
+    float x[kPerWarp][4];
+    const __half* row = p.q + (size_t)m * (p.Hq + 2 * p.Hkv) * kHeadDim + 4 * lane;
+    if constexpr (FUSED) {
+#pragma unroll
+        for (int u = 0; u < kPerWarp; ++u) {
+            const int j = warp + kAttnWarps * u;
+            if (j < G) load4(row + (size_t)(g * G + j) * kHeadDim, x[u]);
+        }
+    }
+    // (a cache of 2^31 tokens would not fit the GPU)
+    const int n = (int)min(min(max(FUSED ? pos + 1 : pos, (int64_t)0), p.L_max),
+                           (int64_t)0x7fffff00);
+    const int nsteps = (n + kStep - 1) / kStep;
+    const int pstep = (int)(pos / kStep);  // fused: the step that holds the new token
+
+    // 16 rows of K and V of step s into ring slot `slot` (zeros past the row's end: a probability
+    // of 0 times garbage could be NaN).  Lane: chunk lane % 16 of rows lane / 16 + 2 u.
+    const uint32_t ring = (uint32_t)__cvta_generic_to_shared(sm.ring[warp]);
+    const size_t lane_off = kv0 + (lane >> 4) * kHeadDim + 8 * (lane & 15);
+    const __half* kl = p.k_cache + lane_off;
+    const __half* vl = p.v_cache + lane_off;
+    auto issue = [&](int s, int slot) {
+        if (s < nsteps) {
+            const uint32_t dst = ring + slot * kStepBytes;
+            const size_t off = (size_t)s * (kStep * kHeadDim);
+            const int left = n - s * kStep;
+#pragma unroll
+            for (int u = 0; u < kStep / 2; ++u) {
+                const int rr = 2 * u + (lane >> 4);
+                const bool ok = rr < left;  // (the first row of a step always exists)
+                const size_t o = off + (ok ? 2 * u * kHeadDim : 0);
+                cp_async16_zfill(dst + swz(rr, lane & 15), kl + o, ok);
+                cp_async16_zfill(dst + kStepBytes / 2 + swz(rr, lane & 15), vl + o, ok);
+            }
         }
         cp_async_commit();
-    }
-    float cs[4], sn[4];
-    rope_angles(lane, p, log2_theta, cs, sn);
-    const __half* row = qkv + (size_t)m * nh * kHeadDim;
-    for (int j = warp; j < G; j += 4) {
-        float x[4], o[4];
-        load4(row + (size_t)(g * G + j) * kHeadDim + 4 * lane, x);
-        norm_rope4(x, qw, lane, cs, sn, eps, o);
-        const uint2 rq = round4(o);  // the fp16 q of the separate path
-        const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&rq.x));
-        const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&rq.y));
-        *reinterpret_cast<float4*>(qs + j * kHeadDim + 4 * lane) =
-            make_float4(scale * a.x, scale * a.y, scale * b.x, scale * b.y);
-    }
+    };
+#pragma unroll
+    for (int i = 0; i < kAttnStages; ++i) issue(wi + i * nw, i);
+
+    // q heads as fp16 rows (zeros past G; rows 4-7 repeat 0-3 unless WIDE); fused: normalised and
+    // rotated here, and the warp that owns the new token's step makes its k and v.
+    const bool holds_new = FUSED && pos >= 0 && pos < p.L_max && pstep % nw == wi;
     uint2 knew = make_uint2(0u, 0u), vnew = make_uint2(0u, 0u);
-    if (holds_new && warp < 2) {
-        if (warp == 0) {
-            float x[4], o[4];
-            load4(row + (size_t)(Hq + g) * kHeadDim + 4 * lane, x);
-            norm_rope4(x, kw, lane, cs, sn, eps, o);
-            knew = round4(o);
-        } else {
-            vnew = *reinterpret_cast<const uint2*>(row + (size_t)(Hq + Hkv + g) * kHeadDim +
-                                                   4 * lane);
+    float xk[4];
+    if (holds_new) {
+        load4(row + (size_t)(p.Hq + g) * kHeadDim, xk);
+        vnew = *reinterpret_cast<const uint2*>(row + (size_t)(p.Hq + p.Hkv + g) * kHeadDim);
+    }
+    if (FUSED && pos != pos_hint) rope_angles(lane, pos, p.log2_theta, cs, sn);
+#pragma unroll
+    for (int u = 0; u < kPerWarp; ++u) {
+        const int j = warp + kAttnWarps * u;
+        uint2 w = make_uint2(0u, 0u);
+        if (j < G) {
+            if constexpr (FUSED) {
+                float o[4];
+                norm_rope4(x[u], p.qw, lane, cs, sn, p.eps, o);
+                w = round4(o);
+            } else {  // (q need not be 8-byte aligned here)
+                const uint16_t* src = reinterpret_cast<const uint16_t*>(p.q) +
+                                      ((size_t)m * p.Hq + g * G + j) * kHeadDim + 4 * lane;
+                w.x = src[0] | (uint32_t)src[1] << 16;
+                w.y = src[2] | (uint32_t)src[3] << 16;
+            }
+        }
+        if (WIDE || j < 4) *reinterpret_cast<uint2*>(sm.q + swz(j, lane >> 1) + 8 * (lane & 1)) = w;
+        if (!WIDE && j < 4)
+            *reinterpret_cast<uint2*>(sm.q + swz(j + 4, lane >> 1) + 8 * (lane & 1)) = w;
+    }
+    if (holds_new) {
+        float o[4];
+        norm_rope4(xk, p.kw, lane, cs, sn, p.eps, o);
+        knew = round4(o);
+    }
+    __syncthreads();
+    uint32_t qb[8][2];  // B fragments of the 8 k16 steps
+    {
+        const uint32_t qs = (uint32_t)__cvta_generic_to_shared(sm.q);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            uint32_t f[4];
+            ldsm4(qs + swz(lane & 7, 4 * t + (lane >> 3)), f);
+            qb[2 * t][0] = f[0];
+            qb[2 * t][1] = f[1];
+            qb[2 * t + 1][0] = f[2];
+            qb[2 * t + 1][1] = f[3];
         }
     }
+
+    const float sl = p.scale * 1.4426950408889634f;  // scores in powers of two
+    // of MMA columns 2c and 2c + 1: scaled max, and this lane's share of sum p
+    float mx[2] = {-INFINITY, -INFINITY}, sum[2] = {0.f, 0.f};
+    // out^T: acc[t][v] is dimension 16 t + r + 8 (v / 2), column 2c + v % 2 (WIDE: acl the low
+    // halves' products)
+    float acc[8][4], acl[WIDE ? 8 : 1][4];
+#pragma unroll
+    for (int t = 0; t < 8; ++t)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) acc[t][v] = acl[WIDE ? t : 0][v] = 0.f;
+
+    const int krow = swz(lane & 15, lane >> 4);  // ldmatrix: tokens lane % 16, chunk lane / 16
+    const int vrow = (((lane >> 4) & 1) * 8 + (lane & 7)) * 256, vj = (lane >> 3) & 1;
+    int slot = 0;
+    for (int s = wi; s < nsteps; s += nw) {
+        cp_async_wait(kAttnStages - 1);
+        __syncwarp();
+        const uint32_t kb = ring + slot * kStepBytes, vb = kb + kStepBytes / 2;
+        if (holds_new && s == pstep) {  // the new token replaces the staged (stale) row
+            const int rr = (int)pos - s * kStep;
+            uint8_t* dst = sm.ring[warp][slot] + swz(rr, lane >> 1) + 8 * (lane & 1);
+            *reinterpret_cast<uint2*>(dst) = knew;
+            *reinterpret_cast<uint2*>(dst + kStepBytes / 2) = vnew;
+            const size_t off = kv0 + (size_t)pos * kHeadDim + 4 * lane;
+            *reinterpret_cast<uint2*>(p.k_cache + off) = knew;
+            *reinterpret_cast<uint2*>(p.v_cache + off) = vnew;
+            __syncwarp();
+        }
+        // scores: sc[v] is token r + 8 (v / 2), column 2c + v % 2 (two chains)
+        float sc[4] = {0.f, 0.f, 0.f, 0.f}, sd[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int ks = 0; ks < 8; ++ks) {
+            uint32_t a[4];
+            ldsm4(kb + (krow ^ (ks << 5)), a);  // chunks 2 ks and 2 ks + 1 of the 16 tokens
+            mma16816(ks & 1 ? sd : sc, a[0], a[1], a[2], a[3], qb[ks][0], qb[ks][1]);
+        }
+        const int left = n - s * kStep;  // (>= 16 in all but the last step)
+        float nm[2];
+        bool grew = false;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            sc[e] = r < left ? sc[e] + sd[e] : -INFINITY;
+            sc[2 + e] = r + 8 < left ? sc[2 + e] + sd[2 + e] : -INFINITY;
+            float v = fmaxf(sc[e], sc[2 + e]);
+            v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 4));
+            v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 8));
+            v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 16)) * sl;
+            nm[e] = fmaxf(mx[e], v);
+            grew |= nm[e] > mx[e];
+        }
+        if (__any_sync(0xffffffffu, grew)) {
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const float f = exp2_diff(mx[e], nm[e]);
+                mx[e] = nm[e];
+                sum[e] *= f;
+#pragma unroll
+                for (int t = 0; t < 8; ++t) {
+                    acc[t][e] *= f;
+                    acc[t][2 + e] *= f;
+                    if (WIDE) {
+                        acl[WIDE ? t : 0][e] *= f;
+                        acl[WIDE ? t : 0][2 + e] *= f;
+                    }
+                }
+            }
+        }
+        uint32_t bh[2], bl[2];  // B fragments: tokens 0-7 and 8-15 of the step
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            float pr[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const float off = (mx[e] == -INFINITY ? 0.f : mx[e]) - 15.f;
+                pr[e] = exp2f(fmaf(sc[2 * t + e], sl, -off));
+                sum[e] += pr[e];
+            }
+            const __half2 h = __floats2half2_rn(pr[0], pr[1]);
+            const float2 hf = __half22float2(h);
+            const __half2 l = __floats2half2_rn(pr[0] - hf.x, pr[1] - hf.y);
+            const uint32_t hw = *reinterpret_cast<const uint32_t*>(&h);
+            const uint32_t lw = *reinterpret_cast<const uint32_t*>(&l);
+            bh[t] = movmatrix(WIDE || c < 2 ? hw : lw);
+            if (WIDE) bl[t] = movmatrix(lw);
+        }
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            uint32_t a[4];  // V^T: dimensions 16 t .. 16 t + 15 of the 16 tokens
+            ldsm4t(vb + vrow + (((2 * t + vj) ^ (lane & 7)) << 4), a);
+            mma16816(acc[t], a[0], a[1], a[2], a[3], bh[0], bh[1]);
+            if (WIDE) mma16816(acl[WIDE ? t : 0], a[0], a[1], a[2], a[3], bl[0], bl[1]);
+        }
+        __syncwarp();  // every lane is done with the slot
+        issue(s + kAttnStages * nw, slot);
+        slot = slot + 1 == kAttnStages ? 0 : slot + 1;
+    }
     asm volatile("cp.async.wait_all;\n" ::: "memory");
-    __syncthreads();
-    if (holds_new && warp < 2) {  // the new token replaces the staged (stale) row
-        const int tt = (int)(p - t0);
-        __half* cache = warp == 0 ? k_cache : v_cache;
-        const uint2 w = warp == 0 ? knew : vnew;
-        *reinterpret_cast<uint2*>(warp == 0 ? &ks[tt][4 * lane] : &vs[tt][4 * lane]) = w;
-        *reinterpret_cast<uint2*>(cache + (kv0 + tt) * kHeadDim + 4 * lane) = w;
+
+    // ---- warps -> CTA (shared memory) ----
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) sum[e] += __shfl_xor_sync(0xffffffffu, sum[e], o);
+        if (r == 0) sm.wml[warp][2 * c + e] = make_float2(mx[e], sum[e]);
+    }
+    __syncthreads();  // (also: every warp is done with its ring)
+    float* red = reinterpret_cast<float*>(&sm.ring[0][0][0]);  // [warp][G][kRedRow]
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const int j = 2 * c + e;  // head
+        float cm = sm.wml[0][j].x;
+#pragma unroll
+        for (int w = 1; w < kAttnWarps; ++w) cm = fmaxf(cm, sm.wml[w][j].x);
+        const float f = exp2_diff(mx[e], cm);
+#pragma unroll
+        for (int t = 0; t < 8; ++t)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const float h = acc[t][2 * u + e];
+                const float l = WIDE ? acl[WIDE ? t : 0][2 * u + e]
+                                     : __shfl_xor_sync(0xffffffffu, h, 2);
+                // (an infinite v times a low half of 0 or of the other sign: the high half alone)
+                if (j < G)
+                    red[(warp * G + j) * kRedRow + 16 * t + 8 * u + r] =
+                        f * (h + (isfinite(l) ? l : 0.f));
+            }
     }
     __syncthreads();
-    chunk_core(ks, vs, qs, sc, mx, sm, nt, G,
-               part + (((size_t)m * Hq + g * G) * nchunk + c) * kPartial, nchunk);
+    const int per = kHeadDim / C;  // dimensions of a CTA's slice
+    cg::cluster_group cluster = cg::this_cluster();
+    if (C > 1) asm volatile("barrier.cluster.wait.aligned;\n" ::: "memory");  // peers have started
+    for (int e = threadIdx.x; e < G * kHeadDim; e += kAttnWarps * 32) {
+        const int j = e / kHeadDim, d = e % kHeadDim;
+        float* recv = C > 1 ? cluster.map_shared_rank(sm.recv, d / per) : sm.recv;
+        float a = 0.f;
+#pragma unroll
+        for (int w = 0; w < kAttnWarps; ++w) a += red[(w * G + j) * kRedRow + d];
+        recv[(rank * G + j) * per + d % per] = a;
+    }
+    for (int u = threadIdx.x; u < C * G; u += kAttnWarps * 32) {
+        const int j = u % G, dst = u / G;
+        float cm = sm.wml[0][j].x, cs = 0.f;
+#pragma unroll
+        for (int w = 1; w < kAttnWarps; ++w) cm = fmaxf(cm, sm.wml[w][j].x);
+#pragma unroll
+        for (int w = 0; w < kAttnWarps; ++w)
+            cs += exp2_diff(sm.wml[w][j].x, cm) * sm.wml[w][j].y;
+        float2* ml = C > 1 ? cluster.map_shared_rank(&sm.ml[0][0], dst) : &sm.ml[0][0];
+        ml[rank * kMaxGroup + j] = make_float2(cm, cs);
+    }
+    // ---- CTAs -> cluster (distributed shared memory), in rank order ----
+    if (C > 1)
+        cluster.sync();
+    else
+        __syncthreads();
+    for (int e = threadIdx.x; e < G * per; e += kAttnWarps * 32) {
+        const int j = e / per, dd = e % per, dim = rank * per + dd;
+        float M = sm.ml[0][j].x;
+        for (int q = 1; q < C; ++q) M = fmaxf(M, sm.ml[q][j].x);
+        float num = 0.f, den = 0.f;
+        for (int q = 0; q < C; ++q) {
+            const float2 ml = sm.ml[q][j];
+            const float f = exp2_diff(ml.x, M);
+            // (a CTA without tokens has f = 0 and partials of 0)
+            num = fmaf(f, sm.recv[(q * G + j) * per + dd], num);
+            den = fmaf(f, ml.y, den);
+        }
+        const size_t h = (size_t)m * p.Hq + g * G + j;
+        if (p.S == 1) {
+            p.out[h * kHeadDim + dim] = __float2half_rn(n == 0 ? 0.f : num / den);
+        } else {
+            float* pp = p.part + (h * p.S + blockIdx.x / C) * kPartial;
+            pp[dim] = num;
+            if (dim == 0) {
+                pp[kHeadDim] = M;
+                pp[kHeadDim + 1] = den;
+            }
+        }
+    }
+}
+
+// Add the partials of the S clusters of each (row, head) in order (maxima in powers of two; a
+// cluster without tokens has max -inf and weight 0).  A row without tokens gets zeros.
+__global__ void __launch_bounds__(kHeadDim) attn_combine_kernel(const float* __restrict__ part,
+                                                                const int32_t* __restrict__ len,
+                                                                int len_is_pos, int Hq, int S,
+                                                                __half* out) {
+    pdl_launch_dependents();
+    pdl_wait();
+    const size_t h = (size_t)blockIdx.y * Hq + blockIdx.x;
+    const float* pp = part + h * S * kPartial;
+    const int d = threadIdx.x;
+    float M = -INFINITY;
+    for (int s = 0; s < S; ++s) M = fmaxf(M, pp[s * kPartial + kHeadDim]);
+    float num = 0.f, den = 0.f;
+    for (int s = 0; s < S; ++s) {
+        const float f = exp2_diff(pp[s * kPartial + kHeadDim], M);
+        num = fmaf(f, pp[s * kPartial + d], num);
+        den = fmaf(f, pp[s * kPartial + kHeadDim + 1], den);
+    }
+    const bool empty = (int64_t)len[blockIdx.y] + (len_is_pos ? 1 : 0) <= 0;
+    out[h * kHeadDim + d] = __float2half_rn(empty ? 0.f : num / den);
 }
 
 // ---- SiLU(gate) * up ----
@@ -606,6 +737,112 @@ laq_status launch_pdl(void (*fn)(KArgs...), dim3 grid, dim3 block, cudaStream_t 
     return e == cudaSuccess ? LAQ_OK : LAQ_ERR_CUDA;
 }
 
+// Clusters of C CTAs per (row, kv head) pair, S clusters per pair.
+//  * C: the most, up to 16 (8 where the device takes no more), that keeps the grid within two CTAs
+//    per SM, the CTAs that are resident together; never more than give each warp one step.
+//    Measured on GB300, fused form, 8 kv heads, 2048 tokens: one row 7.0 / 6.7 us a call at C = 8
+//    / 16; 4 rows 10.9 / 9.9 / 20.1 at C = 4 / 8 / 16; 16 rows 25.0 / 28.7 / 36.7 at C = 2 / 4 / 8.
+//  * S > 1 only where the clusters leave half the SMs idle and a CTA would walk more than 512
+//    tokens: the partials then cost a second launch, less than the walk (one row, 1 kv head: 20.5
+//    -> 12.3 us at 32768 tokens with S = 4, 69 -> 21 us at 131072 with 8; 4 kv heads: 18.4 ->
+//    16.5 us at 16384 with 2; but 8 kv heads, 128 CTAs, 12.9 -> 19 us at 8192 with 2).
+struct AttnShape {
+    int C, S;
+};
+AttnShape attn_shape(int64_t pairs, int64_t L_max, int sms, int max_cluster) {
+    int C = max_cluster;
+    while (C > 1 && pairs * C > 2 * (int64_t)sms) C /= 2;
+    const int64_t steps = (L_max + kStep - 1) / kStep;
+    while (C > 1 && steps <= kAttnWarps * (C / 2)) C /= 2;
+    int64_t S = 1;
+    if (2 * pairs * C <= sms) {
+        const int64_t fill = sms / (pairs * C);
+        const int64_t most = L_max / (512 * (int64_t)C);
+        S = fill < most ? fill : most;
+        if (S < 1) S = 1;
+    }
+    return AttnShape{C, (int)S};
+}
+
+// Once per device and form: the shared-memory limit and the cluster size.  Returns the largest
+// cluster the device schedules (16, or 8), 0 on a CUDA error.
+template <bool FUSED, bool WIDE>
+int attn_setup(int* sms) {
+    static std::atomic<int> cluster_of[64], sms_of[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    int c = cluster_of[dev].load();
+    if (c == 0) {
+        int n = 0;
+        const void* fn = (const void*)attn_kernel<FUSED, WIDE>;
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+            cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(AttnSmem)) != cudaSuccess ||
+            cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 (int)cudaSharedmemCarveoutMaxShared) != cudaSuccess)
+            return 0;
+        c = 8;
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+            cudaSuccess) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(kMaxCluster);
+            cfg.blockDim = dim3(kAttnWarps * 32);
+            cfg.dynamicSmemBytes = sizeof(AttnSmem);
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = kMaxCluster;
+            attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            int fit = 0;
+            if (cudaOccupancyMaxActiveClusters(&fit, fn, &cfg) != cudaSuccess)
+                cudaGetLastError();  // (a refused cluster size is not an error of this call)
+            else if (fit > 0)
+                c = kMaxCluster;
+        } else {
+            cudaGetLastError();
+        }
+        sms_of[dev].store(n);
+        cluster_of[dev].store(c);
+    }
+    *sms = sms_of[dev].load();
+    return c;
+}
+
+template <bool FUSED, bool WIDE>
+laq_status run_attention(AttnParams p, int64_t M, cudaStream_t stream) {
+    int sms = 0;
+    const int max_cluster = attn_setup<FUSED, WIDE>(&sms);
+    if (max_cluster == 0) return LAQ_ERR_CUDA;
+    const AttnShape sh = attn_shape(M * p.Hkv, p.L_max, sms, max_cluster);
+    p.C = sh.C;
+    p.S = sh.S;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(sh.C * sh.S), (unsigned)p.Hkv, (unsigned)M);
+    cfg.blockDim = dim3(kAttnWarps * 32);
+    cfg.dynamicSmemBytes = sizeof(AttnSmem);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)sh.C;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = sh.C > 1 ? 2 : 1;
+    if (cudaLaunchKernelEx(&cfg, attn_kernel<FUSED, WIDE>, p) != cudaSuccess) return LAQ_ERR_CUDA;
+    if (sh.S == 1) return LAQ_OK;
+    return launch_pdl(attn_combine_kernel, dim3((unsigned)p.Hq, (unsigned)M), dim3(kHeadDim),
+                      stream, (const float*)p.part, p.len, FUSED ? 1 : 0, p.Hq, sh.S, p.out);
+}
+
+template <bool FUSED>
+laq_status run_attention(const AttnParams& p, int64_t M, void* stream) {
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    return p.Hq / p.Hkv > 4 ? run_attention<FUSED, true>(p, M, s)
+                            : run_attention<FUSED, false>(p, M, s);
+}
+
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 }  // namespace
@@ -670,17 +907,18 @@ laq_status laq_attention_decode(const void* q, const void* k_cache, const void* 
     if (workspace_bytes < laq_attention_workspace_bytes(M, Hq, L_max)) return LAQ_ERR_WORKSPACE;
     const int64_t nchunk = (L_max + kChunk - 1) / kChunk;
     if (nchunk > 0x7fffffff) return LAQ_ERR_SHAPE;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    laq_status st = launch_pdl(attn_partial_kernel, dim3((unsigned)nchunk, (unsigned)Hkv,
-                                                         (unsigned)M),
-                               dim3(128), s, static_cast<const __half*>(q),
-                               static_cast<const __half*>(k_cache),
-                               static_cast<const __half*>(v_cache), len, (int)Hq, (int)Hkv, L_max,
-                               scale, static_cast<float*>(workspace), (int)nchunk);
-    if (st != LAQ_OK) return st;
-    return launch_pdl(attn_combine_kernel, dim3((unsigned)Hq, (unsigned)M),
-                      dim3(kCombineThreads), s, static_cast<const float*>(workspace), len, 0,
-                      (int)Hq, (int)nchunk, static_cast<__half*>(out));
+    AttnParams p = {};
+    p.q = static_cast<const __half*>(q);
+    p.len = len;
+    p.k_cache = const_cast<__half*>(static_cast<const __half*>(k_cache));  // only read
+    p.v_cache = const_cast<__half*>(static_cast<const __half*>(v_cache));
+    p.out = static_cast<__half*>(out);
+    p.part = static_cast<float*>(workspace);
+    p.L_max = L_max;
+    p.Hq = Hq;
+    p.Hkv = Hkv;
+    p.scale = scale;
+    return run_attention<false>(p, M, stream);
 }
 
 size_t laq_attention_qkv_workspace_bytes(int64_t M, int32_t Hq, int32_t Hkv, int64_t L_max) {
@@ -706,18 +944,22 @@ laq_status laq_attention_qkv(const void* qkv, const void* q_norm_w, const void* 
         return LAQ_ERR_WORKSPACE;
     const int64_t nchunk = (L_max + kChunk - 1) / kChunk;
     if (nchunk > 0x7fffffff) return LAQ_ERR_SHAPE;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    laq_status st = launch_pdl(attn_qkv_kernel, dim3((unsigned)nchunk, (unsigned)Hkv, (unsigned)M),
-                               dim3(128), s, static_cast<const __half*>(qkv),
-                               static_cast<const __half*>(q_norm_w),
-                               static_cast<const __half*>(k_norm_w), pos, (int)Hq, (int)Hkv,
-                               log2f(theta), eps, static_cast<__half*>(k_cache),
-                               static_cast<__half*>(v_cache), L_max, scale,
-                               static_cast<float*>(workspace), (int)nchunk);
-    if (st != LAQ_OK) return st;
-    return launch_pdl(attn_combine_kernel, dim3((unsigned)Hq, (unsigned)M),
-                      dim3(kCombineThreads), s, static_cast<const float*>(workspace), pos, 1,
-                      (int)Hq, (int)nchunk, static_cast<__half*>(out));
+    AttnParams p = {};
+    p.q = static_cast<const __half*>(qkv);
+    p.qw = static_cast<const __half*>(q_norm_w);
+    p.kw = static_cast<const __half*>(k_norm_w);
+    p.len = pos;
+    p.k_cache = static_cast<__half*>(k_cache);
+    p.v_cache = static_cast<__half*>(v_cache);
+    p.out = static_cast<__half*>(out);
+    p.part = static_cast<float*>(workspace);
+    p.L_max = L_max;
+    p.Hq = Hq;
+    p.Hkv = Hkv;
+    p.log2_theta = log2f(theta);
+    p.eps = eps;
+    p.scale = scale;
+    return run_attention<true>(p, M, stream);
 }
 
 laq_status laq_silu_mul(const void* gate_up, int64_t M, int64_t I, void* h, void* stream) {

@@ -132,7 +132,7 @@ class DecodeStep:
                 L.laq_rmsnorm(self.d, nw["in_w"], self.eps, R=self.r, R_out=self.r, Y=self.h,
                               stream=stream)
             self.gemv(self.h, qkv, self.qkv, cf[0], stream, rt.get("qkv"))
-            if self.fused_attention:  # norm, rotation, cache append and attention: two launches
+            if self.fused_attention:  # norm, rotation, cache append and attention: one launch
                 L.laq_attention_qkv(self.qkv, nw["q_w"], nw["k_w"], self.pos, self.Hq, self.Hkv,
                                     self.theta, self.eps, self.kc[l], self.vc[l], self.scale,
                                     self.ws, out=self.att, stream=stream)
@@ -190,11 +190,12 @@ class DecodeStep:
 
     @property
     def launches(self):
-        # embed, norm, per layer 4 GEMVs + 2 norms (1 in layer 0) + attention (2 fused, else
-        # rope + 2) + silu, final norm, LM head, argmax
-        if self.fused_norms:  # embed, per layer 4 GEMVs + 2 attention + silu, norm, LM head, argmax
-            return 1 + self.layers * 7 + 3
-        per_layer = (9 if self.fused_attention else 10) + (4 if self.rotation_rounds else 0)
+        # embed, norm, per layer 4 GEMVs + 2 norms (1 in layer 0) + attention (1 fused, else rope
+        # + 1; one more where a long cache takes the combining launch) + silu, final norm, LM head,
+        # argmax
+        if self.fused_norms:  # embed, per layer 4 GEMVs + attention + silu, norm, LM head, argmax
+            return 1 + self.layers * 6 + 3
+        per_layer = (8 if self.fused_attention else 9) + (4 if self.rotation_rounds else 0)
         return 2 + self.layers * per_layer - 1 + 3
 
     def capture(self, stream=None):
