@@ -443,7 +443,9 @@ def kernel_breakdown(wp, stream, dev, reps=200):
     mp = 1 if wp.M <= 1 else 2 if wp.M <= 2 else 4 if wp.M <= 4 else 8 if wp.M <= 8 else 16
     groups = {}
     for i, (*_, q) in enumerate(wp.linears):
-        key = f"gemm_kernel<{q.bits}, {mp}, {wp.configs[i].tiles_per_cta}>"
+        c = wp.configs[i]
+        key = (f"gemm_batch_kernel<{q.bits}, {1 + (wp.M > 8)}, {c.reserved[1] & 255}>"
+               if c.reserved[0] else f"gemm_kernel<{q.bits}, {mp}, {c.tiles_per_cta}>")
         groups.setdefault(key, []).append(i)
     rows = []
     for key, idxs in groups.items():

@@ -269,6 +269,85 @@ void plan(int64_t M, int64_t K, int64_t N, int bits, int sms, laq_gemm_config* o
     }
 }
 
+// Launch shape of the batch kernel (laq_gemm_batch.cuh), carried in a plan's
+// reserved words beside the general kernel's shape: a tag, and tw | slots << 8 | cluster << 16.
+// A configuration without the tag takes the general kernel.
+constexpr int32_t kBatchTag = 0x4c424154;
+struct BatchShape {
+    int tw, slots, cluster;  // slots = 0: none
+};
+
+BatchShape decode_batch(const laq_gemm_config& c, int64_t M) {
+    BatchShape b{0, 0, 0};
+    if (M < 1 || c.reserved[0] != kBatchTag) return b;
+    const int tw = c.reserved[1] & 255, sl = (c.reserved[1] >> 8) & 255, cl = c.reserved[1] >> 16;
+    if ((tw == 1 || tw == 2) && (sl == 1 || sl == 2 || sl == 4 || sl == 8) && cl >= 1 && cl <= 8)
+        b = BatchShape{tw, sl, cl};
+    return b;
+}
+
+// Shape of the batch kernel: the least estimated time over tiles per warp (1, 2), tile slots per
+// CTA (1..8) and cluster sizes (1..8).  In SM cycles, fitted to 3,700 shapes timed on GB300 (2560 x
+// 6144 .. 2560 x 151936, both widths, M = 3..16; the chosen shape is 2.7 % slower than the best
+// of its sweep on average): a CTA's fixed cost (launch, dependency, reduction), its X by rows and
+// groups, and the group iterations of a warp.  Two CTAs on an SM cost 1.05 x the fixed part and
+// 1.5 x the iterations of one, since one CTA's 8 warps leave latencies exposed; more clusters
+// than can be resident run in waves.  The numbers of CTAs of a cluster size that fit 152 SMs at
+// one and two CTAs per SM are the device's (cudaOccupancyMaxActiveClusters), scaled to `sms`.
+// Lines below as measured inside whole passes (us per layer, general kernel at its plan against
+// this one; every shape swept per projection, the plan within 1 % of the best):
+//  * M = 5..16: always (where a group of X fits): Qwen3-4B W3 M = 8 32.6 -> 28.8, M = 16 49.8 ->
+//    39.3, Qwen3-8B W3 M = 8 65.3 -> 36.9, M = 16 86.4 -> 50.7, a 1408-wide decoder W4 M = 7 17.5
+//    -> 16.3.
+//  * M = 3, 4: K of 32 groups or more with more than 1.5 tiles per SM (Qwen3-8B W4 M = 4 46.0 ->
+//    32.9); the general kernel is faster elsewhere (Qwen3-4B W3 M = 4 24.9, 26.1 with gate|up
+//    here).
+//  * M = 1..4: more than 8 tiles per SM (us per call at W3 M = 1: 2560 x 151936 52.1 -> 38.7, 4096
+//    x 24576 16.0 -> 13.5, 2560 x 32768 13.3 -> 11.9; but 2560 x 19456, 8 tiles per SM, 7.0 ->
+//    7.6).
+void plan_batch(int64_t M, int64_t K, int64_t N, int bits, int sms, laq_gemm_config* out) {
+    static const int kFit[2][8] = {{152, 152, 138, 144, 140, 138, 105, 120},
+                                   {304, 304, 291, 296, 290, 276, 266, 288}};
+    const int64_t T = N / 16, G = K / kGroup;
+    if (M < 1 || T == 0 || G == 0) return;
+    const bool wide = T > 8 * (int64_t)sms;
+    if (M <= 2 && !wide) return;
+    if (M <= 4 && !wide && !(G >= 32 && 2 * T > 3 * (int64_t)sms)) return;
+    const int nb = M > 8 ? 2 : 1;
+    double best = 1e300;
+    for (int tw = 1; tw <= 2; ++tw)
+        for (int sl = 1; sl <= 8; sl *= 2)
+            for (int cl = 1; cl <= 8 && cl <= G; ++cl) {
+                laq::GemmLaunch L;
+                L.M = (int)M;
+                L.K = (int)K;
+                L.N = (int)N;
+                L.bits = bits;
+                L.tw = tw;
+                L.slots = sl;
+                L.cluster = cl;
+                int gpp = 0;
+                if (laq::gemm_batch_smem_bytes(L, &gpp) == 0) continue;
+                const int64_t tc = (int64_t)tw * sl, wk = 8 / sl, gc = (G + cl - 1) / cl;
+                const int64_t ctas = (T + tc - 1) / tc * cl;
+                const int64_t fit1 = (int64_t)kFit[0][cl - 1] * sms / 152;
+                const int64_t fit2 = (int64_t)kFit[1][cl - 1] * sms / 152;
+                const double fixed = 4700.0 + 1600.0 * (double)((gc - 1) / gpp) +
+                                     (double)gc * (29.0 * (double)M + 140.0) +
+                                     6.0 * (double)(tc * M);
+                const double loop = (double)((gc + wk - 1) / wk) *
+                                    (320.0 + tw * (300.0 + 290.0 * (nb - 1)));
+                const int64_t waves = fit2 > 0 ? (ctas + fit2 - 1) / fit2 : ctas;
+                const double cost = ctas <= fit1 ? fixed + loop
+                                                 : (double)waves * (1.05 * fixed + 1.5 * loop);
+                if (cost < best) {
+                    best = cost;
+                    out->reserved[0] = kBatchTag;
+                    out->reserved[1] = tw | sl << 8 | cl << 16;
+                }
+            }
+}
+
 laq_status run_gemm(const void* X, int64_t M, int64_t K, int64_t N, const void* packed,
                     const void* s, const uint8_t* z, int bits, void* Y,
                     const laq_gemm_config* cfg, void* stream,
@@ -303,7 +382,9 @@ laq_status run_gemm(const void* X, int64_t M, int64_t K, int64_t N, const void* 
         c = *cfg;
     } else {
         plan(M, K, N, bits, f.sms, &c);
+        plan_batch(M, K, N, bits, f.sms, &c);
     }
+    const BatchShape b = decode_batch(c, M);
     laq::GemmLaunch L;
     L.X = static_cast<const uint16_t*>(X);
     L.packed = static_cast<const uint8_t*>(packed);
@@ -316,9 +397,11 @@ laq_status run_gemm(const void* X, int64_t M, int64_t K, int64_t N, const void* 
     L.bits = bits;
     L.tiles_per_cta = c.tiles_per_cta;
     L.warps = c.warps;
-    L.cluster = c.cluster;
+    L.cluster = b.slots ? b.cluster : c.cluster;
     L.stages = c.stages;
     L.pdl = c.pdl;
+    L.slots = b.slots;
+    L.tw = b.tw;
     L.pro = kind == LAQ_PROLOGUE_RMSNORM ? laq::kProRmsNorm
             : kind == LAQ_PROLOGUE_SILU_MUL ? laq::kProSiluMul : laq::kProNone;
     if (kind == LAQ_PROLOGUE_RMSNORM) {
@@ -614,6 +697,7 @@ laq_status laq_gemm_plan(int64_t M, int64_t K, int64_t N, int bits, int num_sms,
     if (st != LAQ_OK) return st;
     if (num_sms < 1) return LAQ_ERR_CONFIG;
     plan(M < 1 ? 1 : M, K, N, bits, num_sms, out);
+    plan_batch(M, K, N, bits, num_sms, out);
     return LAQ_OK;
 }
 

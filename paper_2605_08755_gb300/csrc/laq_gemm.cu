@@ -5,7 +5,7 @@
 
 #include <atomic>
 
-#include "laq_gemm_kernel.cuh"
+#include "laq_gemm_batch.cuh"
 
 namespace laq {
 
@@ -16,6 +16,7 @@ int mp_index(int mp) { return mp == 1 ? 0 : mp == 2 ? 1 : mp == 4 ? 2 : mp == 8 
 int nt_index(int nt) { return nt == 1 ? 0 : nt == 2 ? 1 : nt == 4 ? 2 : 3; }
 
 std::atomic<size_t> g_attr_limit[2][2][5][4];  // max dynamic smem granted per kernel instance
+std::atomic<size_t> g_batch_attr_limit[2][2][2][2];
 
 constexpr size_t kXsBudget = 64 * 1024;  // shared memory for staged X (and its tables) per phase
 
@@ -40,17 +41,42 @@ size_t gemm_smem_bytes(const GemmLaunch& L, int* groups_per_phase) {
     return ring + xs + sz + (size_t)L.tiles_per_cta * mp * 16 * 4 + pro;
 }
 
+size_t gemm_batch_smem_bytes(const GemmLaunch& L, int* groups_per_phase) {
+    // two CTAs per SM: half of the SM's 228 KB, less what the hardware reserves per CTA
+    constexpr size_t kHalf = (228 * 1024 - 2 * 1024) / 2;
+    const size_t rec = L.bits == 4 ? 1024 : 768, nb = L.M > 8 ? 2 : 1;
+    const size_t tc = (size_t)L.slots * L.tw, c = (size_t)L.cluster;
+    const size_t units = (tc * L.M + c - 1) / c;
+    const size_t fixed = (size_t)kBatchWarps * kBatchStages * L.tw * rec +
+                         (c > 1 ? c * units * 64 : 0) + (L.pro != kProNone ? 128 : 0);
+    const size_t per_group = nb * (128 * 16 + 8 * 8) + tc * 64;  // X, (S, P), (s, z)
+    if (fixed + per_group > kHalf) return 0;
+    const int gc = (int)((L.K / 128 + c - 1) / c);
+    int gpp = (int)((kHalf - fixed) / per_group);
+    const int phases = (gc + gpp - 1) / gpp;
+    gpp = phases > 0 ? (gc + phases - 1) / phases : 1;  // phases of equal length
+    if (groups_per_phase) *groups_per_phase = gpp;
+    return fixed + (size_t)gpp * per_group;
+}
+
 cudaError_t launch_gemm(const GemmLaunch& L, size_t smem_limit, cudaStream_t stream) {
     int gpp = 1;
-    const size_t smem = gemm_smem_bytes(L, &gpp);
-    if (smem > smem_limit) return cudaErrorInvalidConfiguration;
+    const bool batch = L.slots > 0;
+    const size_t smem = batch ? gemm_batch_smem_bytes(L, &gpp) : gemm_smem_bytes(L, &gpp);
+    if (smem == 0 || smem > smem_limit) return cudaErrorInvalidConfiguration;
     const int mp = mp_class(L.M);
     const bool pro = L.pro != kProNone;
-    const void* fn = pro ? gemm_prologue_kernel(L.bits, mp, L.tiles_per_cta)
-                   : L.bits == 4 ? pick_mp<4, false>(mp, L.tiles_per_cta)
-                                 : pick_mp<3, false>(mp, L.tiles_per_cta);
+    const int nb = L.M > 8 ? 2 : 1;
+    const void* fn =
+        batch ? (pro           ? gemm_batch_prologue_kernel(L.bits, nb, L.tw)
+                 : L.bits == 4 ? pick_batch<4, false>(nb, L.tw)
+                               : pick_batch<3, false>(nb, L.tw))
+        : pro           ? gemm_prologue_kernel(L.bits, mp, L.tiles_per_cta)
+        : L.bits == 4   ? pick_mp<4, false>(mp, L.tiles_per_cta)
+                        : pick_mp<3, false>(mp, L.tiles_per_cta);
     std::atomic<size_t>& granted =
-        g_attr_limit[pro][L.bits == 4][mp_index(mp)][nt_index(L.tiles_per_cta)];
+        batch ? g_batch_attr_limit[pro][L.bits == 4][nb - 1][L.tw - 1]
+              : g_attr_limit[pro][L.bits == 4][mp_index(mp)][nt_index(L.tiles_per_cta)];
     if (granted.load() < smem) {
         // Every instance asks for the largest shared-memory carveout, so kernels of different
         // shapes following each other in a decode step never reconfigure L1 / shared memory.
@@ -63,7 +89,7 @@ cudaError_t launch_gemm(const GemmLaunch& L, size_t smem_limit, cudaStream_t str
         if (e != cudaSuccess) return e;
         granted.store(smem_limit);
     }
-    Params prm;
+    BatchParams prm;  // (the general kernel takes its Params part)
     prm.pro = L.pro;
     prm.eps = L.eps;
     prm.R = L.R;
@@ -81,13 +107,14 @@ cudaError_t launch_gemm(const GemmLaunch& L, size_t smem_limit, cudaStream_t str
     prm.T = L.N / 16;
     prm.stages = L.stages;
     prm.gpp = gpp;
+    prm.slots = L.slots;
     prm.gc = (prm.G + L.cluster - 1) / L.cluster;
     prm.exps = exps_for(L.bits);
 
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((prm.T + L.tiles_per_cta - 1) / L.tiles_per_cta),
-                       (unsigned)L.cluster, 1);
-    cfg.blockDim = dim3((unsigned)(L.warps * 32), 1, 1);
+    const int tc = batch ? L.slots * L.tw : L.tiles_per_cta;
+    cfg.gridDim = dim3((unsigned)((prm.T + tc - 1) / tc), (unsigned)L.cluster, 1);
+    cfg.blockDim = dim3((unsigned)((batch ? kBatchWarps : L.warps) * 32), 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attrs[2];

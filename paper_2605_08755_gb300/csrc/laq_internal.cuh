@@ -22,6 +22,9 @@ struct GemmLaunch {
     uint16_t* Y;
     int M, K, N, bits;
     int tiles_per_cta, warps, cluster, stages, pdl;
+    // batch kernel (laq_gemm_batch.cuh) when slots > 0: tw tiles per warp, slots x tw tiles per
+    // CTA, K over a cluster of `cluster` CTAs (warps, stages and tiles_per_cta unused)
+    int slots = 0, tw = 0;
     // X prologue (kPro*): the GEMV's input is RMSNorm(X + R) * w, or SiLU(gate) * up of X
     int pro = 0;
     float eps = 0.f;
@@ -45,6 +48,8 @@ __host__ __device__ constexpr int xs_row_chunks(int gpp, int mp) {
 // Dynamic shared memory the GEMM kernel needs for this launch (bytes), and the groups of X it
 // stages per phase.
 size_t gemm_smem_bytes(const GemmLaunch& L, int* groups_per_phase);
+// The same for the batch kernel; 0 if one group does not fit half an SM's shared memory.
+size_t gemm_batch_smem_bytes(const GemmLaunch& L, int* groups_per_phase);
 cudaError_t launch_gemm(const GemmLaunch& L, size_t smem_limit, cudaStream_t stream);
 
 // One persistent launch of a GEMV chain, fully resolved on the host.

@@ -1,0 +1,117 @@
+"""The batch kernel at every launch shape it has, on sizes ragged against its tiles,
+teams, clusters and shared-memory phases, and the plan that chooses among them."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import paper_2605_08755_gb300 as laq  # noqa: E402
+from oracle import c_oracle as co  # noqa: E402
+from oracle import decoder as dec  # noqa: E402
+from paper_2605_08755_gb300 import _lib, inputs  # noqa: E402
+
+TAG = 0x4c424154
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    from paper_2605_08755_gb300 import build
+    build.build()
+
+
+def batch_config(tw, slots, cluster, pdl=0):
+    c = laq.GemmConfig.make(1, 8, 1, 4, pdl)
+    c.reserved[0], c.reserved[1] = TAG, tw | slots << 8 | cluster << 16
+    return c
+
+
+def prepared(K, N, bits, seed):
+    W = inputs.weights(K, N, seed=seed)
+    codes, s, z = co.quantize_rtn(W, bits)
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    return ((codes, s, z), dev(co.pack(codes, bits).view(np.uint8)),
+            dev(s.view(np.uint16)).view(torch.float16), dev(z))
+
+
+def check(Y, ref, X, q):
+    """One fp16 rounding, and fp32 sums: a group's accumulator is as large as sum |x_k| times the
+    largest extraction offset (1024) plus the largest code, rounded about 2^-24 of that per
+    addition over 8 MMAs and the start value (16 allowed), times the group's scale."""
+    codes, s, z = q
+    G = s.shape[0]
+    mag = np.abs(X.astype(np.float64)).reshape(X.shape[0], G, 128).sum(-1) * 1040
+    bound = 16 * 2.0 ** -24 * (mag @ s.astype(np.float64)) + 2.0 ** -11 * np.abs(ref) + 2.0 ** -24
+    err = np.abs(Y.astype(np.float64) - ref)
+    assert np.isfinite(Y).all() and (err <= bound).all(), (err / bound).max()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("bits", [3, 4])
+@pytest.mark.parametrize("M", [1, 2, 3, 8, 9, 16])
+def test_every_launch_shape(bits, M):
+    K, N = 1408, 21 * 16     # 11 groups, 21 tiles
+    q, packed, s, z = prepared(K, N, bits, seed=M)
+    X = inputs.activations(M, K, seed=M)
+    ref, xd = co.gemm(X, *q), torch.from_numpy(X).cuda()
+    for tw in (1, 2):
+        for slots in (1, 2, 4, 8):
+            for cluster in range(1, 9):
+                Y = torch.full((M, N), float("nan"), dtype=torch.float16, device="cuda")
+                laq.laq_gemm_wxg128(xd, packed, s, z, bits, Y=Y,
+                                    config=batch_config(tw, slots, cluster, cluster & 1))
+                check(Y.cpu().numpy(), ref, X, q)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("bits", [3, 4])
+@pytest.mark.parametrize("M,K,N,shape", [
+    (16, 128, 16, (2, 8, 1)), (3, 256, 16, (2, 1, 8)),          # fewer groups than CTAs and teams
+    (16, 12288, 272, (2, 8, 1)), (16, 9728, 48, (2, 1, 3)),     # several phases of staged X
+    (5, 16384, 80, (1, 8, 2)), (8, 1920, 1408, (2, 2, 5))])
+def test_phases_and_edges(bits, M, K, N, shape):
+    q, packed, s, z = prepared(K, N, bits, seed=K + N)
+    X = inputs.activations(M, K, seed=K)
+    Y = laq.laq_gemm_wxg128(torch.from_numpy(X).cuda(), packed, s, z, bits,
+                            config=batch_config(*shape))
+    check(Y.cpu().numpy(), co.gemm(X, *q), X, q)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M", [1, 3, 7, 16])
+def test_prologues(M):
+    bits, K, N = 3, 1408, 336
+    q, packed, s, z = prepared(K, N, bits, seed=1)
+    dev = lambda a: torch.from_numpy(a).cuda()
+    x, r = inputs.activations(M, K, seed=2), inputs.activations(M, K, seed=3)
+    w = inputs.norm_weight(K, seed=4)
+    xin, h = dec.rmsnorm(x, w, 1e-6, r)
+    gu = inputs.activations(M, 2 * K, seed=5)
+    for shape in ((2, 4, 1), (1, 2, 3), (2, 8, 8)):
+        cfg = batch_config(*shape)
+        hd = torch.empty((M, K), dtype=torch.float16, device="cuda")
+        Y = _lib.laq_gemm_wxg128_prologue(dev(x), packed, s, z, bits, _lib.PROLOGUE_RMSNORM,
+                                          R=dev(r), R_out=hd, w=dev(w), eps=1e-6, config=cfg)
+        Z = _lib.laq_gemm_wxg128_prologue(dev(gu), packed, s, z, bits, _lib.PROLOGUE_SILU_MUL,
+                                          config=cfg)
+        torch.cuda.synchronize()
+        for y, ref in ((Y, co.gemm(xin, *q)), (Z, co.gemm(dec.silu_mul(gu), *q))):
+            err = np.abs(y.cpu().numpy().astype(np.float64) - ref).max()
+            assert err <= 5e-3 * np.abs(ref).max() + 1e-3  # the GEMV tolerance: inputs round apart
+        assert np.allclose(hd.cpu().numpy().astype(np.float64), h.astype(np.float64), rtol=1e-3,
+                           atol=1e-7)
+
+
+@pytest.mark.parametrize("bits", [3, 4])
+@pytest.mark.parametrize("M", [1, 2, 3, 4, 5, 8, 9, 16])
+def test_plan_names_a_valid_batch_shape(bits, M):
+    for K, N in ((128, 16), (256, 4096), (1408, 7424), (9728, 2560), (4096, 24576), (2560, 151936),
+                 (65535 * 128, 16)):
+        for sms in (152, 1):
+            c = laq.laq_gemm_plan(M, K, N, bits, sms)
+            if M >= 5 or N == 151936:
+                assert c.reserved[0] == TAG
+            if c.reserved[0]:
+                tw, slots, cluster = (c.reserved[1] & 255, c.reserved[1] >> 8 & 255,
+                                      c.reserved[1] >> 16)
+                assert c.reserved[0] == TAG and tw in (1, 2) and slots in (1, 2, 4, 8)
+                assert 1 <= cluster <= min(8, K // 128)
