@@ -348,6 +348,27 @@ void plan_batch(int64_t M, int64_t K, int64_t N, int bits, int sms, laq_gemm_con
             }
 }
 
+// Both plans of a shape, the last few shapes of the thread remembered (a pure function of its
+// arguments; the search over batch shapes takes a few microseconds).
+laq_gemm_config planned(int64_t M, int64_t K, int64_t N, int bits, int sms) {
+    struct Entry {
+        int64_t M, K, N;
+        int bits, sms;
+        laq_gemm_config cfg;
+    };
+    constexpr int kEntries = 16;
+    static thread_local Entry memo[kEntries];  // (zero: M = 0 is never asked for)
+    static thread_local int next = 0;
+    for (const Entry& e : memo)
+        if (e.M == M && e.K == K && e.N == N && e.bits == bits && e.sms == sms) return e.cfg;
+    Entry& e = memo[next];
+    next = (next + 1) % kEntries;
+    e = Entry{M, K, N, bits, sms, {}};
+    plan(M, K, N, bits, sms, &e.cfg);
+    plan_batch(M, K, N, bits, sms, &e.cfg);
+    return e.cfg;
+}
+
 laq_status run_gemm(const void* X, int64_t M, int64_t K, int64_t N, const void* packed,
                     const void* s, const uint8_t* z, int bits, void* Y,
                     const laq_gemm_config* cfg, void* stream,
@@ -381,8 +402,7 @@ laq_status run_gemm(const void* X, int64_t M, int64_t K, int64_t N, const void* 
     if (cfg) {
         c = *cfg;
     } else {
-        plan(M, K, N, bits, f.sms, &c);
-        plan_batch(M, K, N, bits, f.sms, &c);
+        c = planned(M, K, N, bits, f.sms);
     }
     const BatchShape b = decode_batch(c, M);
     laq::GemmLaunch L;
