@@ -296,12 +296,13 @@ BatchShape decode_batch(const laq_gemm_config& c, int64_t M) {
 // one and two CTAs per SM are the device's (cudaOccupancyMaxActiveClusters), scaled to `sms`.
 // Lines below as measured inside whole passes (us per layer, general kernel at its plan against
 // this one; every shape swept per projection, the plan within 1 % of the best):
-//  * M = 5..16: always (where a group of X fits): Qwen3-4B W3 M = 8 32.6 -> 28.8, M = 16 49.8 ->
-//    39.3, Qwen3-8B W3 M = 8 65.3 -> 36.9, M = 16 86.4 -> 50.7, a 1408-wide decoder W4 M = 7 17.5
-//    -> 16.3.
+//  * M = 5..16: always (where a group of X fits): Qwen3-4B W3 M = 8 32.7 -> 26.5, M = 16 49.9 ->
+//    35.0, Qwen3-8B W3 M = 8 65.3 -> 36.9, M = 16 86.2 -> 47.9, a 1408-wide decoder W4 M = 7 17.5
+//    -> 15.8.
 //  * M = 3, 4: K of 32 groups or more with more than 1.5 tiles per SM (Qwen3-8B W4 M = 4 46.0 ->
-//    32.9); the general kernel is faster elsewhere (Qwen3-4B W3 M = 4 24.9, 26.1 with gate|up
-//    here).
+//    32.9), K of 64 groups or more (the 9728 x 2560 down, W3 M = 4 25.0 -> 24.3), and W4 M = 4
+//    from 4 tiles per SM (the 2560 x 19456 gate|up 25.8 -> 25.0; at W3 24.9, 25.1 here).  The
+//    general kernel is as fast or faster on the other Qwen3-4B shapes.
 //  * M = 1..4: more than 8 tiles per SM (us per call at W3 M = 1: 2560 x 151936 52.1 -> 38.7, 4096
 //    x 24576 16.0 -> 13.5, 2560 x 32768 13.3 -> 11.9; but 2560 x 19456, 8 tiles per SM, 7.0 ->
 //    7.6).
@@ -312,7 +313,9 @@ void plan_batch(int64_t M, int64_t K, int64_t N, int bits, int sms, laq_gemm_con
     if (M < 1 || T == 0 || G == 0) return;
     const bool wide = T > 8 * (int64_t)sms;
     if (M <= 2 && !wide) return;
-    if (M <= 4 && !wide && !(G >= 32 && 2 * T > 3 * (int64_t)sms)) return;
+    if (M <= 4 && !wide && !(G >= 32 && 2 * T > 3 * (int64_t)sms) && G < 64 &&
+        !(M == 4 && bits == 4 && T >= 4 * (int64_t)sms))
+        return;
     const int nb = M > 8 ? 2 : 1;
     double best = 1e300;
     for (int tw = 1; tw <= 2; ++tw)

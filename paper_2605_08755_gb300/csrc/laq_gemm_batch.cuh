@@ -13,18 +13,19 @@
 //    (2 KB per 8 rows) and of its (S, P) serves two records;
 //  * X sits in shared memory in fragment order -- chunk 4c + q (x[32c + 8q ..]) of batch row b of
 //    group g at ((g NB + b / 8) 4 + q) 32 + (4 (b % 8) + c), xor 2q -- so a lane's fragment is 4
-//    conflict-free 16-byte loads without address selection, and staging is a plain cp.async of
-//    16-byte chunks (no registers, no shuffles);
+//    conflict-free 16-byte loads without address selection, and staging only moves 16-byte
+//    chunks, four loads in flight per thread (cp.async took 3.9 us for 32 KB per CTA against 1.1;
+//    it queues behind the weight copies);
 //  * S and P come from 8 NB MMAs per group against a constant A (row 0: c_k, row 1: ones), once
 //    per CTA instead of once per staged chunk;
 //  * the accumulator starts at -P - z S, so a group ends with one fma per output: y += s D.
 // 8 warps per CTA, two CTAs per SM: Wt tile slots x Wk = 8 / Wt teams that split the CTA's
 // groups, K split further over a cluster of 1..8 CTAs (any size, so that the grid fills the SMs),
 // reduced through distributed shared memory in rank order.
-// Measured, 4096 x 24576 W3 M = 16, us per call: gemm_kernel 42.9, this one 21.0 (group loop 7.4 of
+// Measured, 4096 x 24576 W3 M = 16, us per call: gemm_kernel 42.9, this one 17.7 (group loop 7.4 of
 // them at 44 SM cycles per record, the rest launch, 45 KB of X per CTA, S and P, reduction).  On
-// the way there: S and P with a conversion instruction and a branch per use 26.0, the reduction
-// with two integer divisions per output 31.2.
+// the way there: X by cp.async 21.0, S and P with a conversion instruction and a branch per use
+// 26.0, the reduction with two integer divisions per output 31.2.
 #pragma once
 #include "laq_gemm_kernel.cuh"
 
@@ -153,18 +154,34 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
             if (PRO && p.pro == kProRmsNorm) rms_rows(p, inv_rms);
             first = false;
         }
-        {   // X of the phase, 16-byte chunks
+        {   // X of the phase, 16-byte chunks, four loads in flight per thread
             const int per_row = ng * 16, nu = M * per_row;  // < 2^16
             const uint32_t inv = 0xffffffffu / (uint32_t)per_row + 1u;
-            for (int u = threadIdx.x; u < nu; u += kBatchWarps * 32) {
-                const int b = (int)__umulhi((uint32_t)u, inv), q = u - b * per_row;
-                const int xo = xb_slot<NB>(q >> 4, b, q & 15);
-                if (PRO) {
-                    xs[xo] = prologue8(p, b, (size_t)pa * 128 + q * 8,
-                                       p.pro == kProRmsNorm ? inv_rms[b] : 0.f);
-                } else {
-                    cp_async16((uint32_t)__cvta_generic_to_shared(xs + xo),
-                               p.X + (size_t)b * p.K + (size_t)pa * 128 + q * 8);
+            constexpr int kFly = PRO ? 2 : 4;
+            for (int u0 = threadIdx.x; u0 < nu; u0 += kFly * kBatchWarps * 32) {
+                uint4 v[kFly], v1[PRO ? kFly : 1];
+#pragma unroll
+                for (int k = 0; k < kFly; ++k) {
+                    const int u = u0 + k * kBatchWarps * 32;
+                    if (u < nu) {
+                        const int b = (int)__umulhi((uint32_t)u, inv), q = u - b * per_row;
+                        const size_t col = (size_t)pa * 128 + q * 8;
+                        if (PRO)
+                            prologue_load(p, b, col, v[k], v1[PRO ? k : 0]);
+                        else
+                            v[k] = ld_cg16(p.X + (size_t)b * p.K + col);
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < kFly; ++k) {
+                    const int u = u0 + k * kBatchWarps * 32;
+                    if (u < nu) {
+                        const int b = (int)__umulhi((uint32_t)u, inv), q = u - b * per_row;
+                        if (PRO)
+                            v[k] = prologue_math(p, (size_t)pa * 128 + q * 8, v[k], v1[PRO ? k : 0],
+                                                 p.pro == kProRmsNorm ? inv_rms[b] : 0.f);
+                        xs[xb_slot<NB>(q >> 4, b, q & 15)] = v[k];
+                    }
                 }
             }
             asm volatile("cp.async.wait_all;\n" ::: "memory");

@@ -116,14 +116,26 @@ __device__ __forceinline__ uint4 pack8f(const float (&f)[8]) {
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// The prologue's transform of the 8 input elements at column k of row b.
-__device__ __forceinline__ uint4 prologue8(const Params& p, int b, size_t k, float inv_rms) {
+// The two loads of the prologue's 8 input elements at column k of row b: X and R (zeros without
+// R), or gate and up.
+__device__ __forceinline__ void prologue_load(const Params& p, int b, size_t k, uint4& v0,
+                                              uint4& v1) {
     if (p.pro == kProRmsNorm) {
-        const uint4 x = ld_cg16(p.X + (size_t)b * p.K + k);
-        const uint4 r = p.R ? ld_cg16(p.R + (size_t)b * p.K + k) : make_uint4(0u, 0u, 0u, 0u);
+        v0 = ld_cg16(p.X + (size_t)b * p.K + k);
+        v1 = p.R ? ld_cg16(p.R + (size_t)b * p.K + k) : make_uint4(0u, 0u, 0u, 0u);
+    } else {
+        v0 = ld_cg16(p.X + (size_t)b * 2 * p.K + k);
+        v1 = ld_cg16(p.X + (size_t)b * 2 * p.K + p.K + k);
+    }
+}
+
+// The prologue's transform of the 8 input elements at column k of a row.
+__device__ __forceinline__ uint4 prologue_math(const Params& p, size_t k, const uint4 v0,
+                                               const uint4 v1, float inv_rms) {
+    if (p.pro == kProRmsNorm) {
         const uint4 wv = *reinterpret_cast<const uint4*>(p.w + k);
         float h[8], y[8];
-        residual8(x, r, h);
+        residual8(v0, v1, h);
         const uint32_t wa[4] = {wv.x, wv.y, wv.z, wv.w};
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -133,9 +145,7 @@ __device__ __forceinline__ uint4 prologue8(const Params& p, int b, size_t k, flo
         }
         return pack8f(y);
     }
-    const uint4 g = ld_cg16(p.X + (size_t)b * 2 * p.K + k);
-    const uint4 u = ld_cg16(p.X + (size_t)b * 2 * p.K + p.K + k);
-    const uint32_t ga[4] = {g.x, g.y, g.z, g.w}, ua[4] = {u.x, u.y, u.z, u.w};
+    const uint32_t ga[4] = {v0.x, v0.y, v0.z, v0.w}, ua[4] = {v1.x, v1.y, v1.z, v1.w};
     // Every CTA of the GEMM recomputes its K range, on the path to the first MMA: the
     // hardware exponential and reciprocal (about 2^-21 relative error, far inside fp16's
     // rounding) cost two special-function operations per element instead of ~40 instructions.
@@ -149,6 +159,12 @@ __device__ __forceinline__ uint4 prologue8(const Params& p, int b, size_t k, flo
         y[2 * i + 1] = __fdividef(a.y, 1.f + __expf(-a.y)) * c.y;
     }
     return pack8f(y);
+}
+
+__device__ __forceinline__ uint4 prologue8(const Params& p, int b, size_t k, float inv_rms) {
+    uint4 v0, v1;
+    prologue_load(p, b, k, v0, v1);
+    return prologue_math(p, k, v0, v1, inv_rms);
 }
 
 // RMSNorm prologue: the inverse RMS of each row of h = fp16(X + R) over its K elements, into
