@@ -116,6 +116,7 @@ __global__ void __launch_bounds__(kRmsThreads) rmsnorm_kernel(const __half* __re
                                                               const __half* __restrict__ w,
                                                               int H, float eps, __half* Y) {
     pdl_launch_dependents();
+    prefetch_l2(w, (size_t)H * 2);
     pdl_wait();
     __shared__ float red[kRmsThreads / 32];
     const size_t row = (size_t)blockIdx.x * H;
@@ -168,6 +169,8 @@ __global__ void __launch_bounds__(128) qk_norm_rope_kernel(
     float log2_theta, float eps, __half* q_out, __half* k_cache, __half* v_cache,
     int64_t L_max) {
     pdl_launch_dependents();
+    prefetch_l2(qw, kHeadDim * 2);
+    prefetch_l2(kw, kHeadDim * 2);
     pdl_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int head = blockIdx.x * 4 + warp, m = blockIdx.y;
@@ -322,7 +325,11 @@ __global__ void __launch_bounds__(kAttnWarps * 32) attn_kernel(const AttnParams 
                 asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p.v_cache + off));
             }
         }
-        if (FUSED) rope_angles(lane, pos_hint, p.log2_theta, cs, sn);
+        if (FUSED) {
+            prefetch_l2(p.qw, kHeadDim * 2);
+            prefetch_l2(p.kw, kHeadDim * 2);
+            rope_angles(lane, pos_hint, p.log2_theta, cs, sn);
+        }
     }
     pdl_wait();
 

@@ -64,6 +64,13 @@ __device__ __forceinline__ uint4 ld_cg16(const void* p) {
     return v;
 }
 
+// Ask L2 for `bytes` from p (128-byte lines, spread over the CTA's threads).  Returns no data, so it
+// may come before pdl_wait() whatever the preceding kernel writes: for parameters that a decode
+// step reads once, whose first touch would otherwise be a DRAM access after the wait.
+__device__ __forceinline__ void prefetch_l2(const void* p, size_t bytes) {
+    for (size_t o = threadIdx.x * 128u; o < bytes; o += blockDim.x * 128u)
+        asm volatile("prefetch.global.L2 [%0];\n" ::"l"(static_cast<const char*>(p) + o));
+}
 __device__ __forceinline__ void pdl_wait() {
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
 }

@@ -74,7 +74,8 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
 
     // shared memory: ring [8][S][TW records] (later the warps' partial sums) | X fragments
     //   [GP][NB][4][32] 16 B | (S, P) [GP][8 NB] float2 | (s, z) [GP][TC][16] half2
-    //   | part [C][UL][16] fp32, UL = ceil(TC M / C) | inv_rms [32] fp32 (prologue)
+    //   | part [C][UL][16] fp32, UL = ceil(TC M / C) | (prologue) inv_rms [16],
+    //   sums of squares by warp [8][16] and by CTA [8][16], fp32
     uint8_t* ring = smem;
     uint4* xs = reinterpret_cast<uint4*>(smem + kBatchWarps * S * kSlot);
     float2* ps = reinterpret_cast<float2*>(xs + (size_t)GP * NB * 128);
@@ -100,6 +101,12 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
 #pragma unroll
             for (int v = 0; v < 4; ++v) yacc[t][h][v] = 0.f;
 
+    // RMSNorm where one phase holds the CTA's whole slice of K (and every CTA has one): X and R are
+    // read once, h = fp16(X + R) is staged, its sums of squares come from the staged fragments and,
+    // over a cluster, from its CTAs, and the staged rows are normalised in place.  (Reading all of X
+    // and R in every CTA for the sums and the slice again for staging: 120 KB per CTA at M = 8, K =
+    // 2560, 4.1 us more per call than a plain GEMM.)
+    const bool in_place = PRO && p.pro == kProRmsNorm && p.gc <= GP && C <= p.G;
     bool first = true;
     for (int pa = g0; pa < g1; pa += GP) {
         const int ng = min(g1, pa + GP) - pa;
@@ -150,8 +157,9 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
             }
         }
         if (first) {
+            if (PRO && p.pro == kProRmsNorm) prefetch_l2(p.w, (size_t)p.K * 2);
             pdl_wait();  // X (and Y) belong to the preceding kernel until it completes
-            if (PRO && p.pro == kProRmsNorm) rms_rows(p, inv_rms);
+            if (PRO && p.pro == kProRmsNorm && !in_place) rms_rows(p, inv_rms);
             first = false;
         }
         {   // X of the phase, 16-byte chunks, four loads in flight per thread
@@ -177,9 +185,15 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
                     const int u = u0 + k * kBatchWarps * 32;
                     if (u < nu) {
                         const int b = (int)__umulhi((uint32_t)u, inv), q = u - b * per_row;
-                        if (PRO)
-                            v[k] = prologue_math(p, (size_t)pa * 128 + q * 8, v[k], v1[PRO ? k : 0],
+                        const size_t col = (size_t)pa * 128 + q * 8;
+                        if (PRO && in_place) {
+                            v[k] = add8h(v[k], v1[PRO ? k : 0]);
+                            if (p.R_out && blockIdx.x == 0)
+                                *reinterpret_cast<uint4*>(p.R_out + (size_t)b * p.K + col) = v[k];
+                        } else if (PRO) {
+                            v[k] = prologue_math(p, col, v[k], v1[PRO ? k : 0],
                                                  p.pro == kProRmsNorm ? inv_rms[b] : 0.f);
+                        }
                         xs[xb_slot<NB>(q >> 4, b, q & 15)] = v[k];
                     }
                 }
@@ -202,6 +216,62 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
                     B[h][2 * q + 1][1] = v.w;
                 }
         };
+        if constexpr (PRO) {
+            if (in_place) {
+                // Sums of squares: the diagonal of H H^T.  A lane's B registers of 8 rows are the A
+                // registers of the same rows too (lane (R, c) holds the same k of row R for both).
+                float d[NB][4];
+#pragma unroll
+                for (int h = 0; h < NB; ++h)
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) d[h][v] = 0.f;
+                for (int lg = warp; lg < ng; lg += kBatchWarps) {
+                    uint32_t B[NB][8][2];
+                    load_b(lg, B);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+#pragma unroll
+                        for (int h = 0; h < NB; ++h)
+                            mma16816(d[h], B[h][j][0], 0u, B[h][j][1], 0u, B[h][j][0], B[h][j][1]);
+                }
+                float* wsum = inv_rms + 16;        // [8 warps][16]
+                float* csum = wsum + 8 * 16;       // [C][16]
+                if (c == R >> 1)  // (row R is column 2c + R % 2 of these lanes)
+#pragma unroll
+                    for (int h = 0; h < NB; ++h) wsum[warp * 16 + 8 * h + R] = R & 1 ? d[h][1] : d[h][0];
+                __syncthreads();
+                if (C > 1)  // every CTA of the cluster has started
+                    asm volatile("barrier.cluster.wait.aligned;\n" ::: "memory");
+                for (int u = threadIdx.x; u < 16 * C; u += kBatchWarps * 32) {
+                    float tot = 0.f;
+#pragma unroll
+                    for (int k = 0; k < kBatchWarps; ++k) tot += wsum[k * 16 + (u & 15)];
+                    float* dst = C > 1 ? cg::this_cluster().map_shared_rank(csum, u >> 4) : csum;
+                    dst[rank * 16 + (u & 15)] = tot;
+                }
+                if (C > 1)
+                    cg::this_cluster().sync();
+                else
+                    __syncthreads();
+                if (threadIdx.x < M) {  // (rows past M hold garbage)
+                    float tot = 0.f;
+                    for (int k = 0; k < C; ++k) tot += csum[k * 16 + threadIdx.x];
+                    inv_rms[threadIdx.x] = rsqrtf(tot / (float)p.K + p.eps);
+                }
+                __syncthreads();
+                const int per_row = ng * 16, nu = M * per_row;
+                const uint32_t inv = 0xffffffffu / (uint32_t)per_row + 1u;
+                for (int u = threadIdx.x; u < nu; u += kBatchWarps * 32) {
+                    const int b = (int)__umulhi((uint32_t)u, inv), q = u - b * per_row;
+                    uint4* x = xs + xb_slot<NB>(q >> 4, b, q & 15);
+                    float h[8];
+                    residual8(*x, make_uint4(0u, 0u, 0u, 0u), h);
+                    *x = rms_apply(h, *reinterpret_cast<const uint4*>(p.w + (size_t)pa * 128 + q * 8),
+                                   inv_rms[b]);
+                }
+                __syncthreads();
+            }
+        }
         // (S, P) of every group and row: MMA row 0 sums c_k x_k, row 1 sums x_k.  A's registers,
         // one per distinct c (bit patterns: a conversion would run at every use).
         uint32_t ca[4];
@@ -311,7 +381,10 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
         }
         asm volatile("cp.async.wait_all;\n" ::: "memory");
     }
-    if (first) pdl_wait();  // a CTA without groups still writes Y after the previous kernel
+    if (first) {  // a CTA without groups still writes Y (and CTA (0, 0) R_out) after the previous kernel
+        pdl_wait();
+        if (PRO && p.pro == kProRmsNorm && p.R_out) rms_rows(p, inv_rms);
+    }
 
     // ---- reduction: teams (shared memory) -> cluster (distributed shared memory) ----
     // Partial sums [8 TW tiles][8 NB rows][16 columns], rows 20 floats apart (the lanes of a store
@@ -346,7 +419,8 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
     cg::cluster_group cluster = cg::this_cluster();
     // Units [r UL, (r + 1) UL) belong to CTA r: every CTA pushes its sums over the teams there, one
     // cluster barrier, then the owner adds the C partials in rank order.
-    if (C > 1) asm volatile("barrier.cluster.wait.aligned;\n" ::: "memory");  // every CTA has started
+    if (C > 1 && !in_place)  // every CTA has started
+        asm volatile("barrier.cluster.wait.aligned;\n" ::: "memory");
     for (int f = threadIdx.x; f < 4 * U; f += kBatchWarps * 32) {
         const int u = f >> 2, q = f & 3, tile = tile_of(u), b = u - tile * M;
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f);

@@ -77,9 +77,10 @@ def test_phases_and_edges(bits, M, K, N, shape):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("M", [1, 3, 7, 16])
-def test_prologues(M):
-    bits, K, N = 3, 1408, 336
+@pytest.mark.parametrize("M,K", [(1, 1408), (3, 1408), (7, 1408), (8, 256), (16, 1408),
+                                 (16, 12288)])   # the last: several phases, two passes over X and R
+def test_prologues(M, K):
+    bits, N = 3, 336
     q, packed, s, z = prepared(K, N, bits, seed=1)
     dev = lambda a: torch.from_numpy(a).cuda()
     x, r = inputs.activations(M, K, seed=2), inputs.activations(M, K, seed=3)
