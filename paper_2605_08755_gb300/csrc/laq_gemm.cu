@@ -49,7 +49,8 @@ size_t gemm_batch_smem_bytes(const GemmLaunch& L, int* groups_per_phase) {
     const size_t units = (tc * L.M + c - 1) / c;
     const size_t fixed = (size_t)kBatchWarps * kBatchStages * L.tw * rec +
                          (c > 1 ? c * units * 64 : 0) + (L.pro != kProNone ? (16 + 8 * 16 + 8 * 16) * 4 : 0);
-    const size_t per_group = nb * (128 * 16 + 8 * 8) + tc * 64;  // X, (S, P), (s, z)
+    const size_t per_group = nb * (128 * 16 + 8 * 8) + tc * 64 +  // X, (S, P), (s, z)
+                             (L.pro != kProNone ? 256 : 0);       // norm weights
     if (fixed + per_group > kHalf) return 0;
     const int gc = (int)((L.K / 128 + c - 1) / c);
     int gpp = (int)((kHalf - fixed) / per_group);

@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
     // shared memory: ring [8][S][TW records] (later the warps' partial sums) | X fragments
     //   [GP][NB][4][32] 16 B | (S, P) [GP][8 NB] float2 | (s, z) [GP][TC][16] half2
     //   | part [C][UL][16] fp32, UL = ceil(TC M / C) | (prologue) inv_rms [16],
-    //   sums of squares by warp [8][16] and by CTA [8][16], fp32
+    //   sums of squares by warp [8][16] and by CTA [8][16], fp32, norm weights [GP][128] fp16
     uint8_t* ring = smem;
     uint4* xs = reinterpret_cast<uint4*>(smem + kBatchWarps * S * kSlot);
     float2* ps = reinterpret_cast<float2*>(xs + (size_t)GP * NB * 128);
@@ -107,6 +107,7 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
     // and R in every CTA for the sums and the slice again for staging: 120 KB per CTA at M = 8, K =
     // 2560, 4.1 us more per call than a plain GEMM.)
     const bool in_place = PRO && p.pro == kProRmsNorm && p.gc <= GP && C <= p.G;
+    uint4* wsm = reinterpret_cast<uint4*>(inv_rms + 16 + 2 * 8 * 16);  // w of the slice
     bool first = true;
     for (int pa = g0; pa < g1; pa += GP) {
         const int ng = min(g1, pa + GP) - pa;
@@ -162,10 +163,14 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
             if (PRO && p.pro == kProRmsNorm && !in_place) rms_rows(p, inv_rms);
             first = false;
         }
-        {   // X of the phase, 16-byte chunks, four loads in flight per thread
+        {   // X of the phase, 16-byte chunks, several loads in flight per thread
             const int per_row = ng * 16, nu = M * per_row;  // < 2^16
             const uint32_t inv = 0xffffffffu / (uint32_t)per_row + 1u;
-            constexpr int kFly = PRO ? 2 : 4;
+            constexpr int kFly = PRO ? 3 : 4;
+            if (PRO && in_place)
+                for (int q = threadIdx.x; q < per_row; q += kBatchWarps * 32)
+                    cp_async16((uint32_t)__cvta_generic_to_shared(wsm + q),
+                               p.w + (size_t)pa * 128 + q * 8);
             for (int u0 = threadIdx.x; u0 < nu; u0 += kFly * kBatchWarps * 32) {
                 uint4 v[kFly], v1[PRO ? kFly : 1];
 #pragma unroll
@@ -266,8 +271,7 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
                     uint4* x = xs + xb_slot<NB>(q >> 4, b, q & 15);
                     float h[8];
                     residual8(*x, make_uint4(0u, 0u, 0u, 0u), h);
-                    *x = rms_apply(h, *reinterpret_cast<const uint4*>(p.w + (size_t)pa * 128 + q * 8),
-                                   inv_rms[b]);
+                    *x = rms_apply(h, wsm[q], inv_rms[b]);
                 }
                 __syncthreads();
             }
