@@ -69,9 +69,8 @@ cudaError_t launch_gemm(const GemmLaunch& L, size_t smem_limit, cudaStream_t str
     const bool pro = L.pro != kProNone;
     const int nb = L.M > 8 ? 2 : 1;
     const void* fn =
-        batch ? (pro           ? gemm_batch_prologue_kernel(L.bits, nb, L.tw)
-                 : L.bits == 4 ? pick_batch<4, false>(nb, L.tw)
-                               : pick_batch<3, false>(nb, L.tw))
+        batch ? (pro ? gemm_batch_prologue_kernel(L.bits, nb, L.tw)
+                     : gemm_batch_plain_kernel(L.bits, nb, L.tw))
         : pro           ? gemm_prologue_kernel(L.bits, mp, L.tiles_per_cta)
         : L.bits == 4   ? pick_mp<4, false>(mp, L.tiles_per_cta)
                         : pick_mp<3, false>(mp, L.tiles_per_cta);

@@ -1,6 +1,6 @@
 // laq_gemm_batch.cuh -- the dequantize-fused GEMM kernel for batches (M = 5..16, and M = 1..4 on
 // wide outputs; the lines stand at plan_batch in laq_api.cu), included by the translation units
-// that instantiate it (laq_gemm.cu: plain X, laq_gemm_prologue.cu: X made by a fused prologue).
+// that instantiate it (laq_gemm_batch.cu: plain X, laq_gemm_prologue.cu: X made by a fused prologue).
 // Same records, extraction and group algebra as laq_gemm_kernel.cuh:
 // D = sum_k (c_k + q_k) x_k on the tensor cores, y += s (D - P - z S) per group, with
 // P = sum_k c_k x_k and S = sum_k x_k.
@@ -465,7 +465,8 @@ const void* pick_batch(int nb, int tw) {
 
 }  // namespace
 
-// The prologue instances (defined in laq_gemm_prologue.cu).
+// The plain-X instances (laq_gemm_batch.cu) and the prologue instances (laq_gemm_prologue.cu).
+const void* gemm_batch_plain_kernel(int bits, int nb, int tw);
 const void* gemm_batch_prologue_kernel(int bits, int nb, int tw);
 
 }  // namespace laq
