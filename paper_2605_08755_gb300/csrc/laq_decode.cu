@@ -673,7 +673,7 @@ __device__ __forceinline__ void better(float& bv, int& bi, float v, int i) {
         bi = i;
     }
 }
-// A cluster of C CTAs per row: CTA r scans the r-th of C equal parts of the row (in whole 8-element
+// A cluster of C (1 or 8) CTAs per row: CTA r scans the r-th of C equal parts of the row (in whole 8-element
 // chunks where the row allows 16-byte loads), sends its candidate to CTA 0, and CTA 0 picks the
 // winner in part order.  Bound: the latency of a dependent launch; one CTA per row took 11 us for
 // a 151,936-entry row (0.3 MB through one SM).  With eight, the head's GEMV + argmax: 67.4 -> 63.4
@@ -1020,10 +1020,11 @@ laq_status laq_argmax(const void* logits, int64_t M, int64_t V, int32_t* out, vo
     if (!logits || !out) return LAQ_ERR_NULL;
     if (M < 1 || M > 65535 || V < 1 || V > 0x7ffffffe) return LAQ_ERR_SHAPE;
     if ((uintptr_t)logits & 1u) return LAQ_ERR_ALIGN;
-    // More CTAs per row while a CTA's part is above 8192 elements (a quarter of a round of its
-    // loads) and the rows leave SMs idle.
-    int C = 1;
-    while (C < 8 && V > (int64_t)65536 / 8 * C && M * C < 128) C *= 2;
+    // A cluster of 8 per row where one CTA would need more than one round of its 32,768-element loads
+    // and few rows leave SMs idle.  Measured on GB300, one CTA against 8, us per call: M = 1, V =
+    // 32768 3.1, 3.6; 49152 4.4, 3.6; 151936 8.1, 3.9; M = 16, V = 65536 4.6, 5.9; 98304 5.9, 6.0;
+    // 151936 8.2, 5.9.
+    const int C = (V > 32768 && M <= 4) || (V > 98304 && M <= 16) ? 8 : 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)C, (unsigned)M);
     cfg.blockDim = dim3(kArgThreads);

@@ -16,8 +16,8 @@ def built():
     build.build()
 
 
-@pytest.mark.parametrize("V", [1, 8, 8191, 8192, 8200, 16392, 32776, 65544, 65537, 151936, 262144])
-@pytest.mark.parametrize("M", [1, 3, 40])
+@pytest.mark.parametrize("V", [1, 8, 8191, 32768, 32776, 49153, 65537, 98312, 151936, 262144])
+@pytest.mark.parametrize("M", [1, 4, 16, 17])
 def test_argmax_parts(V, M):
     rng = np.random.default_rng(V + M)
     x = rng.standard_normal((M, V)).astype(np.float16)
