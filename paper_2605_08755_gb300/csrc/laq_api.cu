@@ -299,22 +299,24 @@ BatchShape decode_batch(const laq_gemm_config& c, int64_t M) {
 //  * M = 5..16: always (where a group of X fits): Qwen3-4B W3 M = 8 32.7 -> 26.5, M = 16 49.9 ->
 //    35.0, Qwen3-8B W3 M = 8 65.3 -> 36.9, M = 16 86.2 -> 47.9, a 1408-wide decoder W4 M = 7 17.5
 //    -> 15.8.
-//  * M = 3, 4: K of 32 groups or more with more than 1.5 tiles per SM (Qwen3-8B W4 M = 4 46.0 ->
-//    32.9), K of 64 groups or more (the 9728 x 2560 down, W3 M = 4 25.0 -> 24.3), and W4 M = 4
+//  * K of 32 groups or more with more than 1.5 tiles per SM, M = 2..4, and M = 1 at W4 (Qwen3-8B,
+//    W3 / W4: M = 1 32.5, 32.5 / 35.5 -> 32.2, M = 2 40.3 -> 33.2 / 42.8 -> 32.1, M = 4 45.6 ->
+//    34.0 / 46.0 -> 32.9).
+//  * M = 3, 4: K of 64 groups or more (the 9728 x 2560 down, W3 M = 4 25.0 -> 24.3), and W4 M = 4
 //    from 4 tiles per SM (the 2560 x 19456 gate|up 25.8 -> 25.0; at W3 24.9, 25.1 here).  The
 //    general kernel is as fast or faster on the other Qwen3-4B shapes.
-//  * M = 1..4: more than 8 tiles per SM (us per call at W3 M = 1: 2560 x 151936 52.1 -> 38.7, 4096
-//    x 24576 16.0 -> 13.5, 2560 x 32768 13.3 -> 11.9; but 2560 x 19456, 8 tiles per SM, 7.0 ->
-//    7.6).
+//  * M = 1..4: more than 8 tiles per SM, 16 at W3 M = 1 (us per call: 2560 x 151936 W3 M = 1 52.1 ->
+//    38.7, M = 3 58.9 -> 41.0; but Qwen3-8B W3 M = 1 with its 10 tiles per SM of gate|up here
+//    33.9 us per layer instead of 32.5).
 void plan_batch(int64_t M, int64_t K, int64_t N, int bits, int sms, laq_gemm_config* out) {
     static const int kFit[2][8] = {{152, 152, 138, 144, 140, 138, 105, 120},
                                    {304, 304, 291, 296, 290, 276, 266, 288}};
     const int64_t T = N / 16, G = K / kGroup;
     if (M < 1 || T == 0 || G == 0) return;
-    const bool wide = T > 8 * (int64_t)sms;
-    if (M <= 2 && !wide) return;
-    if (M <= 4 && !wide && !(G >= 32 && 2 * T > 3 * (int64_t)sms) && G < 64 &&
-        !(M == 4 && bits == 4 && T >= 4 * (int64_t)sms))
+    const bool wide = T > (M == 1 && bits == 3 ? 16 : 8) * (int64_t)sms;
+    const bool big = G >= 32 && 2 * T > 3 * (int64_t)sms;
+    if (!(M >= 5 || wide || (big && (M >= 2 || bits == 4)) ||
+          (M >= 3 && (G >= 64 || (M == 4 && bits == 4 && T >= 4 * (int64_t)sms)))))
         return;
     const int nb = M > 8 ? 2 : 1;
     double best = 1e300;
