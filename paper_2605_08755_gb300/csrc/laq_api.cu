@@ -287,22 +287,24 @@ BatchShape decode_batch(const laq_gemm_config& c, int64_t M) {
 }
 
 // Shape of the batch kernel: the least estimated time over tiles per warp (1, 2), tile slots per
-// CTA (1..8) and cluster sizes (1..8).  In SM cycles, fitted to 3,700 shapes timed on GB300 (2560 x
-// 6144 .. 2560 x 151936, both widths, M = 3..16; the chosen shape is 2.7 % slower than the best
-// of its sweep on average): a CTA's fixed cost (launch, dependency, reduction), its X by rows and
-// groups, and the group iterations of a warp.  Two CTAs on an SM cost 1.05 x the fixed part and
-// 1.5 x the iterations of one, since one CTA's 8 warps leave latencies exposed; more clusters
-// than can be resident run in waves.  The numbers of CTAs of a cluster size that fit 152 SMs at
+// CTA (1..8) and cluster sizes (1..8).  In SM cycles, fitted to sweeps timed on GB300 (16 sizes
+// from 256 x 8192 to 2560 x 151936, both widths, M = 3..16, 4,436 timings; over the 103 sweeps this
+// kernel takes, the chosen shape is 2.7 % slower than the best on average, at most 19 %, 8192 x 512):
+// a CTA's fixed cost (launch, dependency, reduction), its X by rows and groups, and the group
+// iterations of a warp.  Two CTAs on an SM cost 1.05 x the fixed part and 1.5 x the iterations of
+// one, since one CTA's 8 warps leave latencies exposed; more clusters than can be resident run in
+// waves.  The numbers of CTAs of a cluster size that fit 152 SMs at
 // one and two CTAs per SM are the device's (cudaOccupancyMaxActiveClusters), scaled to `sms`.
 // Lines below as measured inside whole passes (us per layer, general kernel at its plan against
-// this one; every shape swept per projection, the plan within 1 % of the best):
-//  * M = 5..16: always (where a group of X fits): Qwen3-4B W3 M = 8 32.7 -> 26.5, M = 16 49.9 ->
-//    35.0, Qwen3-8B W3 M = 8 65.3 -> 36.9, M = 16 86.2 -> 47.9, a 1408-wide decoder W4 M = 7 17.5
+// this plan; the best shapes found by a sweep per projection are up to 3 % faster on Qwen3-4B and
+// Qwen3-8B, 5 % on a 1408-wide decoder):
+//  * M = 5..16: always (where a group of X fits): Qwen3-4B W3 M = 8 32.6 -> 26.6, M = 16 49.9 ->
+//    35.0, Qwen3-8B W3 M = 8 64.9 -> 35.9, M = 16 86.2 -> 47.9, a 1408-wide decoder W4 M = 7 17.5
 //    -> 15.8.
 //  * K of 32 groups or more with more than 1.5 tiles per SM, M = 2..4, and M = 1 at W4 (Qwen3-8B,
-//    W3 / W4: M = 1 32.5, 32.5 / 35.5 -> 32.2, M = 2 40.3 -> 33.2 / 42.8 -> 32.1, M = 4 45.6 ->
-//    34.0 / 46.0 -> 32.9).
-//  * M = 3, 4: K of 64 groups or more (the 9728 x 2560 down, W3 M = 4 25.0 -> 24.3), and W4 M = 4
+//    W4 M = 1 35.3 -> 32.4, W3 / W4 M = 2 40.2 -> 33.6 / 42.7 -> 32.9, M = 4 45.5 -> 34.0 / 45.3 ->
+//    33.0; W3 M = 1 gains nothing, 32.5).
+//  * M = 3, 4: K of 64 groups or more (the 9728 x 2560 down, W3 M = 4 25.1 -> 24.3), and W4 M = 4
 //    from 4 tiles per SM (the 2560 x 19456 gate|up 25.8 -> 25.0; at W3 24.9, 25.1 here).  The
 //    general kernel is as fast or faster on the other Qwen3-4B shapes.
 //  * M = 1..4: more than 8 tiles per SM, 16 at W3 M = 1 (us per call: 2560 x 151936 W3 M = 1 52.1 ->

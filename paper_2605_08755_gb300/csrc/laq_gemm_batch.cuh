@@ -14,18 +14,19 @@
 //  * X sits in shared memory in fragment order -- chunk 4c + q (x[32c + 8q ..]) of batch row b of
 //    group g at ((g NB + b / 8) 4 + q) 32 + (4 (b % 8) + c), xor 2q -- so a lane's fragment is 4
 //    conflict-free 16-byte loads without address selection, and staging only moves 16-byte
-//    chunks, four loads in flight per thread (cp.async took 3.9 us for 32 KB per CTA against 1.1;
-//    it queues behind the weight copies);
+//    chunks, four loads in flight per thread (cp.async queues behind the weight copies: 3.9 us
+//    for 32 KB per CTA against 1.1, median CTA of a tracing build);
 //  * S and P come from 8 NB MMAs per group against a constant A (row 0: c_k, row 1: ones), once
 //    per CTA instead of once per staged chunk;
 //  * the accumulator starts at -P - z S, so a group ends with one fma per output: y += s D.
 // 8 warps per CTA, two CTAs per SM: Wt tile slots x Wk = 8 / Wt teams that split the CTA's
 // groups, K split further over a cluster of 1..8 CTAs (any size, so that the grid fills the SMs),
 // reduced through distributed shared memory in rank order.
-// Measured, 4096 x 24576 W3 M = 16, us per call: gemm_kernel 42.9, this one 17.7 (group loop 7.4 of
-// them at 44 SM cycles per record, the rest launch, 45 KB of X per CTA, S and P, reduction).  On
-// the way there: X by cp.async 21.0, S and P with a conversion instruction and a branch per use
-// 26.0, the reduction with two integer divisions per output 31.2.
+// Measured, us per call in a chain of calls: 4096 x 24576 W3 M = 16 gemm_kernel 42.9, this one 19.9;
+// 2560 x 19456 W3 M = 8 10.8, 9.1; 9728 x 2560 W4 M = 4 6.7, 6.4.  Of the first, the group loop takes
+// 8.6 in the median CTA, the rest is launch, 45 KB of X per CTA, S and P, reduction.  Its first
+// version took 31.2 (S and P with conversions and branches, integer divisions in the reduction),
+// 20.9 without those, and the rest of the way came with plain loads of X.
 #pragma once
 #include "laq_gemm_kernel.cuh"
 
@@ -105,7 +106,7 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
     // read once, h = fp16(X + R) is staged, its sums of squares come from the staged fragments and,
     // over a cluster, from its CTAs, and the staged rows are normalised in place.  (Reading all of X
     // and R in every CTA for the sums and the slice again for staging: 120 KB per CTA at M = 8, K =
-    // 2560, 4.1 us more per call than a plain GEMM.)
+    // 2560, 4.2 us more per call than a plain GEMM; in place about 3.)
     const bool in_place = PRO && p.pro == kProRmsNorm && p.gc <= GP && C <= p.G;
     uint4* wsm = reinterpret_cast<uint4*>(inv_rms + 16 + 2 * 8 * 16);  // w of the slice
     bool first = true;
