@@ -18,7 +18,12 @@
 //    for 32 KB per CTA against 1.1, median CTA of a tracing build);
 //  * S and P come from 8 NB MMAs per group against a constant A (row 0: c_k, row 1: ones), once
 //    per CTA instead of once per staged chunk;
-//  * the accumulator starts at -P - z S, so a group ends with one fma per output: y += s D.
+//  * D and P are two accumulator chains each (even and odd k16 steps) from zero, in the same order:
+//    the tensor core truncates every sum at the magnitude of the running value (up to 1024 sum |x|),
+//    so halves that stay half as long, and a P whose truncation follows D's, leave less in D - P.
+//    Error against 64 bits beyond the final fp16 rounding, W4 2560 x 19456 M = 16, N(0, 1) X: 2.8e-5
+//    of the result (gemm_kernel, with P by fp32 additions, 2.8e-5; one chain started at -P - z S
+//    4.6e-5, one chain from zero 4.3e-5); with 1 % outliers of 50 in X 2.0e-5, 3.6e-5, 6.7e-5, 2.9e-5.
 // 8 warps per CTA, two CTAs per SM: Wt tile slots x Wk = 8 / Wt teams that split the CTA's
 // groups, K split further over a cluster of 1..8 CTAs (any size, so that the grid fills the SMs),
 // reduced through distributed shared memory in rank order.
@@ -288,17 +293,19 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
         for (int lg = warp; lg < ng; lg += kBatchWarps) {
             uint32_t B[NB][8][2];
             load_b(lg, B);
-            float d[NB][4];
+            float d[2][NB][4];
 #pragma unroll
-            for (int h = 0; h < NB; ++h)
+            for (int a = 0; a < 2; ++a)
 #pragma unroll
-                for (int v = 0; v < 4; ++v) d[h][v] = 0.f;
+                for (int h = 0; h < NB; ++h)
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) d[a][h][v] = 0.f;
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const int k0 = offset_index<BITS>(2 * j), k1 = offset_index<BITS>(2 * j + 1);
 #pragma unroll
                 for (int h = 0; h < NB; ++h)
-                    mma16816(d[h], ca[k0], 0u, ca[k1], 0u, B[h][j][0], B[h][j][1]);
+                    mma16816(d[j & 1][h], ca[k0], 0u, ca[k1], 0u, B[h][j][0], B[h][j][1]);
             }
             if (R < 2) {
 #pragma unroll
@@ -306,7 +313,7 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
                         float* dst = reinterpret_cast<float*>(ps + (lg * NB + h) * 8 + 2 * c + e);
-                        dst[R == 0 ? 1 : 0] = d[h][e];
+                        dst[R == 0 ? 1 : 0] = d[0][h][e] + d[1][h][e];
                     }
             }
         }
@@ -356,26 +363,30 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
                     const uint32_t w = szp[16 * t + 8 * r];
                     szv[r] = __half22float2(*reinterpret_cast<const __half2*>(&w));
                 }
-                float D[NB][4];
+                float D[2][NB][4];
 #pragma unroll
-                for (int h = 0; h < NB; ++h)
+                for (int e = 0; e < 2; ++e)
 #pragma unroll
-                    for (int r = 0; r < 2; ++r) {
-                        D[h][2 * r] = fmaf(-szv[r].y, sp[h].x, -sp[h].y);
-                        D[h][2 * r + 1] = fmaf(-szv[r].y, sp[h].z, -sp[h].w);
-                    }
+                    for (int h = 0; h < NB; ++h)
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) D[e][h][v] = 0.f;
                 uint32_t a[8][4];
                 extract<BITS>(wd, p.exps, a);
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
 #pragma unroll
                     for (int h = 0; h < NB; ++h)
-                        mma16816(D[h], a[j][0], a[j][1], a[j][2], a[j][3], B[h][j][0], B[h][j][1]);
+                        mma16816(D[j & 1][h], a[j][0], a[j][1], a[j][2], a[j][3], B[h][j][0],
+                                 B[h][j][1]);
 #pragma unroll
                 for (int h = 0; h < NB; ++h)
 #pragma unroll
-                    for (int v = 0; v < 4; ++v)
-                        yacc[t][h][v] = fmaf(szv[v >> 1].x, D[h][v], yacc[t][h][v]);
+                    for (int v = 0; v < 4; ++v) {  // y += s (D - P - z S)
+                        const float S_ = v & 1 ? sp[h].z : sp[h].x, P_ = v & 1 ? sp[h].w : sp[h].y;
+                        const float d = D[0][h][v] + D[1][h][v] - P_;
+                        yacc[t][h][v] =
+                            fmaf(szv[v >> 1].x, fmaf(-szv[v >> 1].y, S_, d), yacc[t][h][v]);
+                    }
             }
 #pragma unroll
             for (int q = 0; q < 4; ++q) xq[q] += Wk * NB * 128;

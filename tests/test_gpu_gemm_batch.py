@@ -64,6 +64,34 @@ def test_every_launch_shape(bits, M):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("bits", [3, 4])
+@pytest.mark.parametrize("K", [1408, 4096])
+@pytest.mark.parametrize("outliers", [False, True])
+def test_sums_are_as_exact_as_the_general_kernels(bits, K, outliers):
+    """What a kernel adds to the final fp16 rounding, over 16 batches: the batch kernel's no more
+    than the general kernel's.  A row's groups share their P, so the errors of a row go together:
+    256 rows make the root mean square good to about 5 %, two of them to 7; 1.15 is twice that.
+    (One accumulator chain started at -P - z S: 1.5 times the general kernel's, 2.1 with outliers.)"""
+    M, N = 16, 1024
+    q, packed, s, z = prepared(K, N, bits, seed=K)
+    own = {}
+    for seed in range(16):
+        X = inputs.activations(M, K, seed=seed).astype(np.float32)
+        if outliers:
+            X[np.random.default_rng(seed).random(X.shape) < 0.01] *= 50
+        X = X.astype(np.float16)
+        ref = co.gemm(X, *q)
+        rounded = ref.astype(np.float16)
+        for name, cfg in (("batch", batch_config(2, 4, 1)),
+                          ("general", laq.GemmConfig.make(8, 8, 1, 4))):
+            Y = laq.laq_gemm_wxg128(torch.from_numpy(X).cuda(), packed, s, z, bits, config=cfg)
+            d2 = np.square(Y.cpu().numpy().astype(np.float64) - ref)
+            own[name] = own.get(name, 0.0) + (
+                (d2 - np.square(rounded.astype(np.float64) - ref)).sum() / np.square(ref).sum())
+    assert 0 < own["batch"] <= 1.15 ** 2 * own["general"], (own["batch"] / own["general"]) ** 0.5
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("bits", [3, 4])
 @pytest.mark.parametrize("M,K,N,shape", [
     (16, 128, 16, (2, 8, 1)), (3, 256, 16, (2, 1, 8)),          # fewer groups than CTAs and teams
     (16, 12288, 272, (2, 8, 1)), (16, 9728, 48, (2, 1, 3)),     # several phases of staged X
