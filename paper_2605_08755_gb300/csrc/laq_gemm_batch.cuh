@@ -229,27 +229,38 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
         };
         if constexpr (PRO) {
             if (in_place) {
-                // Sums of squares: the diagonal of H H^T.  A lane's B registers of 8 rows are the A
-                // registers of the same rows too (lane (R, c) holds the same k of row R for both).
-                float d[NB][4];
+                // Sums of squares in fp32 (the tensor core truncates: on it 20 % of the rows at K =
+                // 4096 had every input rounded as by 64 bits, here and in gemm_kernel 80 %).  A lane
+                // of a group's fragments holds 32 of the 128 elements of row 8h + R.
+                float d[NB];
 #pragma unroll
-                for (int h = 0; h < NB; ++h)
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) d[h][v] = 0.f;
+                for (int h = 0; h < NB; ++h) d[h] = 0.f;
                 for (int lg = warp; lg < ng; lg += kBatchWarps) {
                     uint32_t B[NB][8][2];
                     load_b(lg, B);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j)
+                    for (int h = 0; h < NB; ++h) {
+                        float e0 = 0.f, e1 = 0.f;
 #pragma unroll
-                        for (int h = 0; h < NB; ++h)
-                            mma16816(d[h], B[h][j][0], 0u, B[h][j][1], 0u, B[h][j][0], B[h][j][1]);
+                        for (int j = 0; j < 8; ++j)
+#pragma unroll
+                            for (int k = 0; k < 2; ++k) {
+                                const float2 f =
+                                    __half22float2(*reinterpret_cast<const __half2*>(&B[h][j][k]));
+                                e0 = fmaf(f.x, f.x, e0);
+                                e1 = fmaf(f.y, f.y, e1);
+                            }
+                        d[h] += e0 + e1;
+                    }
                 }
                 float* wsum = inv_rms + 16;        // [8 warps][16]
                 float* csum = wsum + 8 * 16;       // [C][16]
-                if (c == R >> 1)  // (row R is column 2c + R % 2 of these lanes)
 #pragma unroll
-                    for (int h = 0; h < NB; ++h) wsum[warp * 16 + 8 * h + R] = R & 1 ? d[h][1] : d[h][0];
+                for (int h = 0; h < NB; ++h) {
+                    d[h] += __shfl_xor_sync(0xffffffffu, d[h], 1);
+                    d[h] += __shfl_xor_sync(0xffffffffu, d[h], 2);
+                    if (c == 0) wsum[warp * 16 + 8 * h + R] = d[h];
+                }
                 __syncthreads();
                 if (C > 1)  // every CTA of the cluster has started
                     asm volatile("barrier.cluster.wait.aligned;\n" ::: "memory");
