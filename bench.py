@@ -444,8 +444,8 @@ def kernel_breakdown(wp, stream, dev, reps=200):
     groups = {}
     for i, (*_, q) in enumerate(wp.linears):
         c = wp.configs[i]
-        key = (f"gemm_batch_kernel<{q.bits}, {1 + (wp.M > 8)}, {c.reserved[1] & 255}>"
-               if c.reserved[0] else f"gemm_kernel<{q.bits}, {mp}, {c.tiles_per_cta}>")
+        key = (f"gemm_batch_kernel<{q.bits}, {1 + (wp.M > 8)}, {c.batch[0]}>"
+               if c.batch else f"gemm_kernel<{q.bits}, {mp}, {c.tiles_per_cta}>")
         groups.setdefault(key, []).append(i)
     rows = []
     for key, idxs in groups.items():

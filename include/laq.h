@@ -158,10 +158,10 @@ typedef struct {
     int32_t cluster;
     int32_t stages;
     int32_t pdl;
-    int32_t reserved[3]; /* 0, or as laq_gemm_plan set them: the launch shape of the batch kernel,
-                            which then replaces tiles_per_cta, warps, cluster and
-                            stages; those describe the general kernel, which serves every other
-                            configuration */
+    int32_t reserved[3]; /* 0: the general kernel runs, in the shape of the fields above.  As
+                            laq_gemm_plan set them: the batch kernel runs, in a shape of its own, as
+                            long as tiles_per_cta, warps, cluster and stages are also as planned; a
+                            plan with one of these four changed runs the general kernel so */
 } laq_gemm_config;
 
 /* The configuration laq_gemm_wxg128 uses for this shape on a GPU with `num_sms` SMs (host-only

@@ -40,13 +40,36 @@ class GemmConfig(ctypes.Structure):
                 ("cluster", ctypes.c_int32), ("stages", ctypes.c_int32), ("pdl", ctypes.c_int32),
                 ("reserved", ctypes.c_int32 * 3)]
 
+    BATCH_TAG = 0x4c424154  # reserved[0] of a configuration that names a batch kernel shape
+
+    def _general_shape(self):
+        return self.tiles_per_cta | self.warps << 8 | self.cluster << 16 | self.stages << 24
+
+    @property
+    def batch(self):
+        """(tiles per warp, tile slots per CTA, cluster) of the batch kernel if this configuration
+        runs it, None if it runs the general kernel."""
+        tag, shape, planned = self.reserved
+        if tag != self.BATCH_TAG or planned not in (0, self._general_shape()):
+            return None
+        return shape & 255, shape >> 8 & 255, shape >> 16
+
     def as_dict(self):
-        return {"tiles_per_cta": self.tiles_per_cta, "warps": self.warps,
-                "cluster": self.cluster, "stages": self.stages, "pdl": self.pdl}
+        """The arguments of ``make`` that give this configuration."""
+        d = {"tiles_per_cta": self.tiles_per_cta, "warps": self.warps,
+             "cluster": self.cluster, "stages": self.stages, "pdl": self.pdl}
+        if self.batch:
+            d["batch"] = self.batch
+        return d
 
     @classmethod
-    def make(cls, tiles_per_cta, warps, cluster, stages, pdl=0):
-        return cls(tiles_per_cta, warps, cluster, stages, pdl, (ctypes.c_int32 * 3)(0, 0, 0))
+    def make(cls, tiles_per_cta, warps, cluster, stages, pdl=0, batch=None):
+        c = cls(tiles_per_cta, warps, cluster, stages, pdl, (ctypes.c_int32 * 3)(0, 0, 0))
+        if batch:
+            tw, slots, batch_cluster = batch
+            c.reserved[:] = (cls.BATCH_TAG, tw | slots << 8 | batch_cluster << 16,
+                             c._general_shape())
+        return c
 
 
 class GemmPrologue(ctypes.Structure):

@@ -269,17 +269,23 @@ void plan(int64_t M, int64_t K, int64_t N, int bits, int sms, laq_gemm_config* o
     }
 }
 
-// Launch shape of the batch kernel (laq_gemm_batch.cuh), carried in a plan's
-// reserved words beside the general kernel's shape: a tag, and tw | slots << 8 | cluster << 16.
-// A configuration without the tag takes the general kernel.
+// Launch shape of the batch kernel (laq_gemm_batch.cuh), carried in a plan's reserved words beside
+// the general kernel's shape: a tag, tw | slots << 8 | cluster << 16, and the general shape it was
+// planned with (0: any).  A configuration without the tag, or whose general shape was changed since,
+// takes the general kernel.
 constexpr int32_t kBatchTag = 0x4c424154;
 struct BatchShape {
     int tw, slots, cluster;  // slots = 0: none
 };
 
+int32_t general_shape(const laq_gemm_config& c) {
+    return c.tiles_per_cta | c.warps << 8 | c.cluster << 16 | c.stages << 24;  // (checked: <= 16)
+}
+
 BatchShape decode_batch(const laq_gemm_config& c, int64_t M) {
     BatchShape b{0, 0, 0};
     if (M < 1 || c.reserved[0] != kBatchTag) return b;
+    if (c.reserved[2] != 0 && c.reserved[2] != general_shape(c)) return b;
     const int tw = c.reserved[1] & 255, sl = (c.reserved[1] >> 8) & 255, cl = c.reserved[1] >> 16;
     if ((tw == 1 || tw == 2) && (sl == 1 || sl == 2 || sl == 4 || sl == 8) && cl >= 1 && cl <= 8)
         b = BatchShape{tw, sl, cl};
@@ -351,6 +357,7 @@ void plan_batch(int64_t M, int64_t K, int64_t N, int bits, int sms, laq_gemm_con
                     best = cost;
                     out->reserved[0] = kBatchTag;
                     out->reserved[1] = tw | sl << 8 | cl << 16;
+                    out->reserved[2] = general_shape(*out);
                 }
             }
 }

@@ -4,8 +4,10 @@ For one fused 36-layer pass (q|k|v, o, gate|up, down; Qwen3-4B or Qwen3-8B shape
 batch rows M) captured as one CUDA graph, every launch shape (tiles per CTA, warps, cluster)
 of one projection type is tried in turn -- the other projections keep the library's plan, the
 ring depth follows the library's rule for the shape -- and the pass is timed (CUDA events on
-the replaying stream, best of three runs of 100 replays).  Prints the library's shape and the
-fastest shapes for each projection type, then the pass with every type at its fastest.
+the replaying stream, best of three runs of 100 replays).  Prints the library's plan and the
+fastest shapes for each projection type, then the pass with every type at its fastest.  The shapes
+tried are the general kernel's; where the plan names the batch kernel (its line then shows that
+shape), a fastest shape above the plan's time says by how much the batch kernel wins.
 
     python -m paper_2605_08755_gb300.measure.shape_sweep --model qwen3-8b --bits 3 --M 1
 """
@@ -60,9 +62,7 @@ def main():
         return t
 
     def config(q, nt, w, cl, st):
-        c = _lib.laq_gemm_plan(a.M, q.K, q.N, a.bits, sms)
-        c.tiles_per_cta, c.warps, c.cluster, c.stages, c.pdl = nt, w, cl, st, 1
-        return c
+        return _lib.GemmConfig.make(nt, w, cl, st, 1)  # the general kernel
 
     out = {"model": a.model, "bits": a.bits, "M": a.M, "library_us": timed(base), "types": {}}
     print(f"{a.model} W{a.bits} M={a.M}: library plan {out['library_us']:.1f} us per pass",
@@ -86,9 +86,9 @@ def main():
                 continue   # more shared memory than a CTA may have
         res.sort()
         b = base[idx[0]]
-        lib = (b.tiles_per_cta, b.warps, b.cluster, b.stages)
+        lib = b.batch or (b.tiles_per_cta, b.warps, b.cluster, b.stages)
         out["types"][ty] = {"K": q.K, "N": q.N, "library": lib, "timings": res}
-        print(f"  {ty:8s} K={q.K:5d} N={q.N:5d} library {lib}  fastest "
+        print(f"  {ty:8s} K={q.K:5d} N={q.N:5d} library {'batch ' if b.batch else ''}{lib}  fastest "
               + ", ".join(f"{r[0]:.1f} {tuple(r[1:4])}" for r in res[:4]),
               flush=True)
         best[ty] = (q, res[0])

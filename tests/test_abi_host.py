@@ -224,7 +224,10 @@ def test_plan_shares_x_across_tiles_above_m_two(L):
             assert laq.laq_gemm_plan(2, K, N, bits, 152).as_dict() == one(K, N, bits)
         for M in (3, 4):
             # the long-K down projection keeps the M = 1 shape (4-warp CTAs of 2 tiles, cluster 8)
-            assert laq.laq_gemm_plan(M, 9728, 2560, bits, 152).as_dict() == one(9728, 2560, bits)
+            # (the general kernel's; which kernel runs is the batch plan's choice)
+            c = laq.laq_gemm_plan(M, 9728, 2560, bits, 152).as_dict()
+            c.pop("batch", None)
+            assert c == one(9728, 2560, bits)
             # otherwise X shared by 4 tiles per CTA, K split until about one CTA per SM
             assert shape(laq.laq_gemm_plan(M, 2560, 6144, bits, 152))[:3] == (4, 8, 2)
             assert shape(laq.laq_gemm_plan(M, 4096, 2560, bits, 152))[:3] == (4, 8, 4)
