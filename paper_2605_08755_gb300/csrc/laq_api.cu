@@ -37,10 +37,11 @@ laq_status from_cuda(cudaError_t e) {
 
 // Per-device facts the planner and launcher need, cached on first use.
 struct DeviceFacts {
+    int device;
     int sms;
     size_t smem_optin;
 };
-constexpr int kMaxDevices = 64;
+using laq::kMaxDevices;
 std::atomic<int> g_sms[kMaxDevices];
 std::atomic<long long> g_smem[kMaxDevices];
 
@@ -62,6 +63,7 @@ laq_status device_facts(DeviceFacts* f) {
         g_sms[dev].store(sms);
         g_smem[dev].store(smem);
     }
+    f->device = dev;
     f->sms = sms;
     f->smem_optin = (size_t)smem;
     return LAQ_OK;
@@ -436,6 +438,7 @@ laq_status run_gemm(const void* X, int64_t M, int64_t K, int64_t N, const void* 
     L.pdl = c.pdl;
     L.slots = b.slots;
     L.tw = b.tw;
+    L.device = f.device;
     L.pro = kind == LAQ_PROLOGUE_RMSNORM ? laq::kProRmsNorm
             : kind == LAQ_PROLOGUE_SILU_MUL ? laq::kProSiluMul : laq::kProNone;
     if (kind == LAQ_PROLOGUE_RMSNORM) {
@@ -560,6 +563,7 @@ laq_status run_chain(const laq_gemv* g, int32_t count, void* workspace, size_t w
     L.bits = bits;
     L.xs_bytes = (int)xs_need;
     L.ws = static_cast<uint32_t*>(workspace);
+    L.device = f.device;
     if (use_static && cudaMemsetAsync(workspace, 0, laq::chain_workspace_zeroed_bytes(count),
                                       static_cast<cudaStream_t>(stream)) != cudaSuccess)
         return LAQ_ERR_CUDA;

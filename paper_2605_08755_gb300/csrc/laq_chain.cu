@@ -746,7 +746,8 @@ ChainFn pick_chain(int mp) {
     }
 }
 
-std::atomic<size_t> g_chain_attr[2][3];  // dynamic shared memory already granted per instance
+// dynamic shared memory already granted per device and instance
+std::atomic<size_t> g_chain_attr[kMaxDevices][2][3];
 
 }  // namespace
 
@@ -785,7 +786,8 @@ cudaError_t launch_chain(const ChainLaunch& L, int num_sms, cudaStream_t stream)
     const int mp = L.M <= 1 ? 1 : L.M <= 2 ? 2 : 4;
     const ChainFn fn = L.bits == 4 ? pick_chain<4>(mp) : pick_chain<3>(mp);
     const size_t smem = chain_smem_bytes(L.bits, L.M, L.xs_bytes, L.nstages, L.count);
-    std::atomic<size_t>& granted = g_chain_attr[L.bits == 4][mp == 1 ? 0 : mp == 2 ? 1 : 2];
+    std::atomic<size_t>& granted =
+        g_chain_attr[L.device][L.bits == 4][mp == 1 ? 0 : mp == 2 ? 1 : 2];
     cudaError_t err = cudaSuccess;
     if (granted.load() < smem) {
         err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

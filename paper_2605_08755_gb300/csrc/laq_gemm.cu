@@ -15,8 +15,9 @@ int mp_class(int M) { return M <= 1 ? 1 : M <= 2 ? 2 : M <= 4 ? 4 : M <= 8 ? 8 :
 int mp_index(int mp) { return mp == 1 ? 0 : mp == 2 ? 1 : mp == 4 ? 2 : mp == 8 ? 3 : 4; }
 int nt_index(int nt) { return nt == 1 ? 0 : nt == 2 ? 1 : nt == 4 ? 2 : 3; }
 
-std::atomic<size_t> g_attr_limit[2][2][5][4];  // max dynamic smem granted per kernel instance
-std::atomic<size_t> g_batch_attr_limit[2][2][2][2];
+// max dynamic smem granted per device and kernel instance
+std::atomic<size_t> g_attr_limit[kMaxDevices][2][2][5][4];
+std::atomic<size_t> g_batch_attr_limit[kMaxDevices][2][2][2][2];
 
 constexpr size_t kXsBudget = 64 * 1024;  // shared memory for staged X (and its tables) per phase
 
@@ -75,8 +76,8 @@ cudaError_t launch_gemm(const GemmLaunch& L, size_t smem_limit, cudaStream_t str
         : L.bits == 4   ? pick_mp<4, false>(mp, L.tiles_per_cta)
                         : pick_mp<3, false>(mp, L.tiles_per_cta);
     std::atomic<size_t>& granted =
-        batch ? g_batch_attr_limit[pro][L.bits == 4][nb - 1][L.tw - 1]
-              : g_attr_limit[pro][L.bits == 4][mp_index(mp)][nt_index(L.tiles_per_cta)];
+        batch ? g_batch_attr_limit[L.device][pro][L.bits == 4][nb - 1][L.tw - 1]
+              : g_attr_limit[L.device][pro][L.bits == 4][mp_index(mp)][nt_index(L.tiles_per_cta)];
     if (granted.load() < smem) {
         // Every instance asks for the largest shared-memory carveout, so kernels of different
         // shapes following each other in a decode step never reconfigure L1 / shared memory.

@@ -5,6 +5,8 @@
 
 namespace laq {
 
+constexpr int kMaxDevices = 64;  // what is remembered per device holds for ordinals below this
+
 // Exactly one of codes and packed is given.
 cudaError_t launch_quantize(const uint16_t* W, int64_t K, int64_t N, int bits, uint8_t* codes,
                             uint8_t* packed, uint16_t* s, uint8_t* z, cudaStream_t stream);
@@ -22,6 +24,7 @@ struct GemmLaunch {
     uint16_t* Y;
     int M, K, N, bits;
     int tiles_per_cta, warps, cluster, stages, pdl;
+    int device = 0;  // the current device (function attributes are per device)
     // batch kernel (laq_gemm_batch.cuh) when slots > 0: tw tiles per warp, slots x tw tiles per
     // CTA, K over a cluster of `cluster` CTAs (warps, stages and tiles_per_cta unused)
     int slots = 0, tw = 0;
@@ -77,6 +80,7 @@ struct ChainLaunch {
     const ChainStage* st;
     int count, nstages, M, bits, xs_bytes;
     uint32_t* ws;
+    int device;  // the current device
 };
 // Dynamic shared memory of the chain kernel (its ring depth is fixed per bit width).
 size_t chain_smem_bytes(int bits, int M, int xs_bytes, int nstages, int count);

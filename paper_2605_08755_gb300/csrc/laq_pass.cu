@@ -49,6 +49,7 @@
 
 #include "laq.h"
 #include "laq_device.cuh"
+#include "laq_internal.cuh"
 
 namespace laq {
 namespace {
@@ -1070,7 +1071,8 @@ __global__ void pass_gather_kernel(const GatherRec* __restrict__ gt,
     }
 }
 
-std::atomic<int> g_pass_attr[2][3];  // shared memory granted to pass_kernel<bits, 1 | 2 | 4>
+// shared memory granted, by device, to pass_kernel<bits, 1 | 2 | 4>
+std::atomic<int> g_pass_attr[kMaxDevices][2][3];
 
 template <int BITS>
 const void* pick_pass(int mp) {
@@ -1078,9 +1080,10 @@ const void* pick_pass(int mp) {
                    : mp == 2 ? (const void*)pass_kernel<BITS, 2> : (const void*)pass_kernel<BITS, 4>;
 }
 
-int device_sms(int* sms, int* smem_optin) {
+int device_sms(int* device, int* sms, int* smem_optin) {
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return -1;
+    *device = dev;
     if (cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return -1;
     if (cudaDeviceGetAttribute(smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
@@ -1172,8 +1175,8 @@ laq_status laq_pass_run(const void* plan, const void* device, void* workspace,
     if ((reinterpret_cast<uintptr_t>(workspace) & 15u) || workspace_bytes < pass_workspace(*h))
         return LAQ_ERR_WORKSPACE;
     if (h->nstages == 0) return LAQ_OK;
-    int sms = 0, optin = 0;
-    if (device_sms(&sms, &optin) != 0) return LAQ_ERR_CUDA;
+    int ordinal = 0, sms = 0, optin = 0;
+    if (device_sms(&ordinal, &sms, &optin) != 0) return LAQ_ERR_CUDA;
     if (sms != h->sms) return LAQ_ERR_CONFIG;  // planned for another SM count
     // ring depth: as many 16-record slots as the shared memory left over holds
     const int mp = h->M == 1 ? 1 : h->M == 2 ? 2 : 4;
@@ -1208,7 +1211,7 @@ laq_status laq_pass_run(const void* plan, const void* device, void* workspace,
     const void* fn = h->bits == 4 ? pick_pass<4>(mp) : pick_pass<3>(mp);
     // First call with this much shared memory (before any stream capture): raise the kernel's
     // limit and check that a CTA fits an SM, as the cooperative launch requires.
-    std::atomic<int>& granted = g_pass_attr[h->bits == 4][mp == 1 ? 0 : mp == 2 ? 1 : 2];
+    std::atomic<int>& granted = g_pass_attr[ordinal][h->bits == 4][mp == 1 ? 0 : mp == 2 ? 1 : 2];
     if (granted.load() < L.total) {
         if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, L.total) !=
             cudaSuccess)

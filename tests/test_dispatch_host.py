@@ -31,7 +31,8 @@ def F(tmp_path_factory):
                    + objs, check=True)
     L = ctypes.CDLL(so)
     real = _lib.lib()
-    for name in ("laq_gemm_wxg128", "laq_gemm_wxg128_config", "laq_gemm_wxg128_prologue"):
+    for name in ("laq_gemm_wxg128", "laq_gemm_wxg128_config", "laq_gemm_wxg128_prologue",
+                 "laq_gemm_chain", "laq_pass_run"):
         getattr(L, name).argtypes = getattr(real, name).argtypes
     L.fake_last_kernel.restype = ctypes.c_char_p
     return L
@@ -79,3 +80,41 @@ def test_a_plan_survives_its_dictionary(F, M):
         again = laq.GemmConfig.make(**c.as_dict())
         assert bytes(again) == bytes(c)
         assert gemm(F, again, M, K, N, 3) == gemm(F, c, M, K, N, 3)
+
+
+def entries(M, dims):
+    arr = (_lib.Gemv * len(dims))()
+    for i, (K, N) in enumerate(dims):
+        arr[i] = _lib.Gemv(FAKE, FAKE, FAKE, FAKE, FAKE, M, K, N, 3, 1)
+    return arr
+
+
+@pytest.mark.parametrize("what", ["general", "batch", "norm", "chain", "pass"])
+def test_every_device_is_granted_shared_memory(F, what):
+    """Function attributes hold for one device: the second GPU of a process asks for its own."""
+    ws = ctypes.c_void_p(0x200000)
+    dims = [(4096, 4096), (4096, 2560)]
+
+    def run():
+        if what == "chain":
+            return F.laq_gemm_chain(entries(1, dims), 2, ws, 1 << 20, None)
+        if what == "pass":
+            plan, _ = _lib.pass_plan(entries(1, dims), 2, SMS)
+            return F.laq_pass_run(plan, ctypes.c_void_p(0x100000), ws, 1 << 20, None)
+        M = 1 if what == "general" else 16
+        cfg = laq.laq_gemm_plan(M, 4096, 24576, 3, SMS)
+        assert (cfg.batch is None) == (what == "general")
+        if what == "norm":
+            pro = _lib.GemmPrologue(_lib.PROLOGUE_RMSNORM, 1e-6, None, None, FAKE)
+            return F.laq_gemm_wxg128_prologue(FAKE, M, 4096, 24576, FAKE, FAKE, FAKE, 3, FAKE,
+                                              ctypes.byref(pro), ctypes.byref(cfg), None)
+        return F.laq_gemm_wxg128_config(FAKE, M, 4096, 24576, FAKE, FAKE, FAKE, 3, FAKE,
+                                        ctypes.byref(cfg), None)
+    try:
+        for device in (0, 1, 0):
+            F.fake_set_device(device)
+            n = F.fake_launches()
+            assert (run(), F.fake_launches() - n) == (0, 1), device
+            assert launched(F)[5] > 48 * 1024
+    finally:
+        F.fake_set_device(0)
