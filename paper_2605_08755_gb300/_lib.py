@@ -230,14 +230,13 @@ def laq_gemm_wxg128(X, packed, s, z, bits, Y=None, config=None, stream=None):
         import torch
         Y = X.new_empty((M, N), dtype=torch.float16)
     if config is None:
-        st = lib().laq_gemm_wxg128(X.data_ptr(), M, K, N, packed.data_ptr(), s.data_ptr(),
-                                   z.data_ptr(), bits, Y.data_ptr(), _stream(stream))
+        st = lib().laq_gemm_wxg128(_ptr(X), M, K, N, _ptr(packed), _ptr(s), _ptr(z), bits, _ptr(Y),
+                                   _stream(stream))
         if st:
             _check(st, "laq_gemm_wxg128")
     else:
-        st = lib().laq_gemm_wxg128_config(X.data_ptr(), M, K, N, packed.data_ptr(), s.data_ptr(),
-                                          z.data_ptr(), bits, Y.data_ptr(), ctypes.byref(config),
-                                          _stream(stream))
+        st = lib().laq_gemm_wxg128_config(_ptr(X), M, K, N, _ptr(packed), _ptr(s), _ptr(z), bits,
+                                          _ptr(Y), ctypes.byref(config), _stream(stream))
         if st:
             _check(st, "laq_gemm_wxg128_config")
     return Y

@@ -108,6 +108,18 @@ def test_gemm_config_validation(L):
                                     None) == 1
 
 
+@pytest.mark.parametrize("config", [None, laq.GemmConfig.make(1, 2, 1, 2)])
+def test_binding_refuses_a_missing_tensor(L, config):
+    torch = pytest.importorskip("torch")
+    t = dict(X=torch.zeros((1, 128), dtype=torch.float16), packed=torch.zeros(1, dtype=torch.uint8),
+             s=torch.zeros((1, 16), dtype=torch.float16), z=torch.zeros((1, 16), dtype=torch.uint8))
+    stream = type("Stream", (), {"cuda_stream": 0})()
+    for name in ("packed", "z"):
+        with pytest.raises(laq.LaqError) as e:
+            laq.laq_gemm_wxg128(**{**t, name: None}, bits=3, config=config, stream=stream)
+        assert e.value.status == 1, name
+
+
 def test_quantize_pack_argument_validation(L):
     q = L.laq_quantize_rtn
     assert q(FAKE, 256, 32, 3, 64, FAKE, FAKE, FAKE, None) == 3
