@@ -19,6 +19,7 @@
 
 #include "laq.h"
 #include "laq_device.cuh"
+#include "laq_internal.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -297,8 +298,10 @@ __device__ __forceinline__ float exp2_diff(float a, float b) {  // 2^(a - b); a 
     return a == -INFINITY ? 0.f : exp2f(a - b);
 }
 
+// Two CTAs per SM, as attn_shape counts on (the copies' addresses below cost the WIDE form 156
+// registers when the compiler is left free, 128 and no spills with the bound).
 template <bool FUSED, bool WIDE>
-__global__ void __launch_bounds__(kAttnWarps * 32) attn_kernel(const AttnParams p) {
+__global__ void __launch_bounds__(kAttnWarps * 32, 2) attn_kernel(const AttnParams p) {
     pdl_launch_dependents();
     if (p.C > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");
     extern __shared__ __align__(128) uint8_t attn_smem[];
@@ -353,9 +356,8 @@ __global__ void __launch_bounds__(kAttnWarps * 32) attn_kernel(const AttnParams 
     // 16 rows of K and V of step s into ring slot `slot` (zeros past the row's end: a probability
     // of 0 times garbage could be NaN).  Lane: chunk lane % 16 of rows lane / 16 + 2 u.
     const uint32_t ring = (uint32_t)__cvta_generic_to_shared(sm.ring[warp]);
-    const size_t lane_off = kv0 + (lane >> 4) * kHeadDim + 8 * (lane & 15);
-    const __half* kl = p.k_cache + lane_off;
-    const __half* vl = p.v_cache + lane_off;
+    const __half* kl = p.k_cache + kv0;
+    const __half* vl = p.v_cache + kv0;
     auto issue = [&](int s, int slot) {
         if (s < nsteps) {
             const uint32_t dst = ring + slot * kStepBytes;
@@ -364,8 +366,8 @@ __global__ void __launch_bounds__(kAttnWarps * 32) attn_kernel(const AttnParams 
 #pragma unroll
             for (int u = 0; u < kStep / 2; ++u) {
                 const int rr = 2 * u + (lane >> 4);
-                const bool ok = rr < left;  // (the first row of a step always exists)
-                const size_t o = off + (ok ? 2 * u * kHeadDim : 0);
+                const bool ok = rr < left;
+                const size_t o = off + attn_copy_offset(lane, u, left);
                 cp_async16_zfill(dst + swz(rr, lane & 15), kl + o, ok);
                 cp_async16_zfill(dst + kStepBytes / 2 + swz(rr, lane & 15), vl + o, ok);
             }

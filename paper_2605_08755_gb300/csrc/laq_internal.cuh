@@ -55,6 +55,13 @@ size_t gemm_smem_bytes(const GemmLaunch& L, int* groups_per_phase);
 size_t gemm_batch_smem_bytes(const GemmLaunch& L, int* groups_per_phase);
 cudaError_t launch_gemm(const GemmLaunch& L, size_t smem_limit, cudaStream_t stream);
 
+// Attention: the 16-byte chunk that a lane copies for row 2u + lane / 16 of a 16-token step of which
+// `left` >= 1 rows exist, in elements from the step's first row (rows of 128).  Past the last row the
+// copy is of no bytes (the row is filled with zeros) and its address that of the step's first row.
+__host__ __device__ constexpr int attn_copy_offset(int lane, int u, int left) {
+    return (2 * u + (lane >> 4) < left ? 2 * u + (lane >> 4) : 0) * 128 + 8 * (lane & 15);
+}
+
 // One persistent launch of a GEMV chain, fully resolved on the host.
 constexpr int kChainMax = 384;  // = LAQ_CHAIN_MAX
 struct ChainEntry {

@@ -16,6 +16,11 @@ FAKE = ctypes.c_void_p(0x10000)   # never dereferenced
 SMS = 152
 
 
+def cuda_include():
+    nvcc = os.path.realpath(build._nvcc())
+    return os.path.join(os.path.dirname(os.path.dirname(nvcc)), "include")
+
+
 @pytest.fixture(scope="module")
 def F(tmp_path_factory):
     build.build()
@@ -23,9 +28,8 @@ def F(tmp_path_factory):
     objs = [os.path.join(build.BUILD_DIR, s.replace(".cu", ".o")) for s in build.SOURCES]
     if not all(os.path.exists(o) for o in objs):
         build.build(force=True)
-    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build._nvcc()))), "include")
     obj, so = str(d / "fake.o"), str(d / "liblaq_fake.so")
-    subprocess.run([shutil.which("gcc"), "-O1", "-fPIC", "-I", inc, "-c",
+    subprocess.run([shutil.which("gcc"), "-O1", "-fPIC", "-I", cuda_include(), "-c",
                     os.path.join(ROOT, "tests", "fake_cudart.c"), "-o", obj], check=True)
     subprocess.run([shutil.which("g++"), "-shared", "-Wl,-Bsymbolic", "-Wl,-z,defs", "-o", so, obj]
                    + objs, check=True)
@@ -118,3 +122,33 @@ def test_every_device_is_granted_shared_memory(F, what):
             assert launched(F)[5] > 48 * 1024
     finally:
         F.fake_set_device(0)
+
+
+def test_attention_copies_stay_inside_the_step(tmp_path):
+    """Every address a copy of a step is given, also one of no bytes past the row's last token, lies
+    in rows that exist: in a cache filled to its last row the next one is past the allocation."""
+    src = tmp_path / "offsets.cpp"
+    src.write_text("""
+#include <cuda_runtime.h>
+#include <stdint.h>
+#include <cstdio>
+#include "laq_internal.cuh"
+int main() {
+    for (int left = 1; left <= 16; ++left) {
+        bool seen[16 * 16] = {};
+        for (int lane = 0; lane < 32; ++lane)
+            for (int u = 0; u < 8; ++u) {
+                const int o = laq::attn_copy_offset(lane, u, left);
+                if (o < 0 || o % 8 || o + 8 > left * 128) return 1;
+                if (2 * u + lane / 16 < left) seen[o / 8] = true;
+            }
+        for (int j = 0; j < left * 16; ++j)
+            if (!seen[j]) return 2;
+    }
+    return 0;
+}
+""")
+    exe = str(tmp_path / "offsets")
+    subprocess.run([shutil.which("g++"), "-std=c++17", "-I", cuda_include(), "-I", build.CSRC, "-o",
+                    exe, str(src)], check=True)
+    assert subprocess.run([exe]).returncode == 0
