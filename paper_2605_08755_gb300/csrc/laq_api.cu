@@ -294,40 +294,56 @@ BatchShape decode_batch(const laq_gemm_config& c, int64_t M) {
     return b;
 }
 
+// Whether the batch kernel takes a shape (t = tiles per SM), as timed on GB300 by
+// measure/kernel_choice.py, us: chains of dependent calls of one size (ratio general / batch kernel
+// in their planned shapes) and whole decoder layers.
+//  * M = 5..16: always.  Chains 0.97 to 2.9 (M = 5..8, 512 or 1024 columns and 28 groups or more 0.90 to
+//    0.98, calls of 3.4 to 3.8 us); Qwen3-4B W3 M = 8 31.8 -> 26.1 us per layer, M = 16 48.4 -> 34.5,
+//    Qwen3-8B W3 M = 8 64.1 -> 36.9, M = 16 85.3 -> 48.8, a 1408-wide decoder W4 M = 8 16.6 -> 15.5.
+//  * M = 3, 4, t > 8: always (1.0 to 2.2).  M = 2, t > 8: K of 16 groups (W4: 11) or more, 0.99 to
+//    1.6; below, 0.74 to 1.1.  M = 1, t > 8, W4: 18 groups or more, 1.02 to 1.5; below, 0.72 to
+//    1.5.  M = 1, W3: t > 24 and 16 groups or more, 1.06 to 1.38 (2560 x 151936 52.1 -> 38.7 us); up to
+//    t = 24, 0.72 to 1.3, and the Qwen3-8B gate|up (t = 10) 33.9 us per layer here, 32.5 there.
+//  * K of 32 groups or more, t > 1.5, M = 2..4: 0.90 to 2.0 in chains (9728 columns at M = 2, W3 0.84);
+//    the sizes below 1 (t <= 4 and K under 40 groups) gain where their neighbours run this kernel too:
+//    Qwen3-8B M = 2 39.4 -> 34.6 us per layer (W4 43.2 -> 34.2), 35.4 with the general kernel for its
+//    4096 x 4096.  M = 1, W4: t > 4 or K of 64 groups, 0.95 to 1.6 (Qwen3-8B 35.9 -> 33.9); below 0.77
+//    to 0.95.
+//  * K of 72 groups or more, M = 3, 4, narrower outputs: t >= 1.25 from 64 groups 1.34 to 1.6; t >=
+//    0.5 from 88 groups 1.03 to 1.33; t >= 1 from 72 groups at M = 4 and W4 M = 3, 1.02 to 1.1
+//    (Qwen3-4B M = 4 24.1 -> 23.8 us per layer); below 0.88 to 1.0.
+//  * M = 4, W4, t > 4, K of 20 groups or more: 1.1 to 1.8 (Qwen3-4B with its gate|up here 24.05 us per
+//    layer, 24.6 without); shorter K 0.65 to 1.0.
+bool batch_takes(int64_t M, int64_t G, int64_t T, int bits, int64_t sms) {
+    if (M >= 5) return true;
+    const bool w4 = bits == 4;
+    if (M == 1 && !w4) return T > 24 * sms && G >= 16;
+    if (T > 8 * sms && G >= (M == 1 ? 18 : M == 2 ? (w4 ? 11 : 16) : 1)) return true;
+    if (G >= 32 && 2 * T > 3 * sms && (M >= 2 || T > 4 * sms || G >= 64)) return true;
+    if (M < 3) return false;
+    if (G >= 64 && 4 * T >= 5 * sms) return true;
+    if (G >= 88 && 2 * T >= sms) return true;
+    if (G >= 72 && T >= sms && (M == 4 || w4)) return true;
+    return M == 4 && w4 && T > 4 * sms && G >= 20;
+}
+
 // Shape of the batch kernel: the least estimated time over tiles per warp (1, 2), tile slots per
-// CTA (1..8) and cluster sizes (1..8).  In SM cycles, fitted to sweeps timed on GB300 (16 sizes
-// from 256 x 8192 to 2560 x 151936, both widths, M = 3..16, 4,436 timings; over the 103 sweeps this
-// kernel takes, the chosen shape is 2.7 % slower than the best on average, at most 19 %, 8192 x 512):
-// a CTA's fixed cost (launch, dependency, reduction), its X by rows and groups, and the group
-// iterations of a warp.  Two CTAs on an SM cost 1.05 x the fixed part and 1.5 x the iterations of
-// one, since one CTA's 8 warps leave latencies exposed; more clusters than can be resident run in
-// waves.  The numbers of CTAs of a cluster size that fit 152 SMs at
-// one and two CTAs per SM are the device's (cudaOccupancyMaxActiveClusters), scaled to `sms`.
-// Lines below as measured inside whole passes (us per layer, general kernel at its plan against
-// this plan; the best shapes found by a sweep per projection are up to 3 % faster on Qwen3-4B and
-// Qwen3-8B, 5 % on a 1408-wide decoder):
-//  * M = 5..16: always (where a group of X fits): Qwen3-4B W3 M = 8 32.6 -> 26.6, M = 16 49.9 ->
-//    35.0, Qwen3-8B W3 M = 8 64.9 -> 35.9, M = 16 86.2 -> 47.9, a 1408-wide decoder W4 M = 7 17.5
-//    -> 15.8.
-//  * K of 32 groups or more with more than 1.5 tiles per SM, M = 2..4, and M = 1 at W4 (Qwen3-8B,
-//    W4 M = 1 35.3 -> 32.4, W3 / W4 M = 2 40.2 -> 33.6 / 42.7 -> 32.9, M = 4 45.5 -> 34.0 / 45.3 ->
-//    33.0; W3 M = 1 gains nothing, 32.5).
-//  * M = 3, 4: K of 64 groups or more (the 9728 x 2560 down, W3 M = 4 25.1 -> 24.3), and W4 M = 4
-//    from 4 tiles per SM (the 2560 x 19456 gate|up 25.8 -> 25.0; at W3 24.9, 25.1 here).  The
-//    general kernel is as fast or faster on the other Qwen3-4B shapes.
-//  * M = 1..4: more than 8 tiles per SM, 16 at W3 M = 1 (us per call: 2560 x 151936 W3 M = 1 52.1 ->
-//    38.7, M = 3 58.9 -> 41.0; but Qwen3-8B W3 M = 1 with its 10 tiles per SM of gate|up here
-//    33.9 us per layer instead of 32.5).
+// CTA (1..8) and cluster sizes (1..8).  In SM cycles, fitted to sweeps of all shapes in chains of
+// calls (measure/kernel_choice.py --shapes): a CTA's fixed cost (launch, dependency, reduction), its X
+// by rows and groups, and the group iterations of a warp.  Two CTAs on an SM cost 1.05 x the fixed
+// part and 1.5 x the iterations of one, since one CTA's 8 warps leave latencies exposed; with
+// clusters of 7 or 8 that leave a CTA 2 groups, or 3 of up to one tile per SM, 1.3 x the fixed part,
+// which is then most of the call (whole layers of a 1024-wide decoder W4 M = 8 15.5 -> 13.5 us,
+// 2048-wide 20.0 -> 19.2; with 1.3 for longer slices too, a 1408-wide decoder's 16 layers at M = 7 went
+// 253 -> 260 us, and a 3072-wide one with its 3 groups of 192 tiles 33.9 -> 34.5 us per layer).  More
+// clusters than can be resident run in waves.  The numbers of CTAs of a cluster size that fit 152 SMs
+// at one and two CTAs per SM are the device's (cudaOccupancyMaxActiveClusters), scaled to `sms`.
+// X is taken as given: an RMSNorm prologue whose slice then needs two phases reads X and R twice.
 void plan_batch(int64_t M, int64_t K, int64_t N, int bits, int sms, laq_gemm_config* out) {
     static const int kFit[2][8] = {{152, 152, 138, 144, 140, 138, 105, 120},
                                    {304, 304, 291, 296, 290, 276, 266, 288}};
     const int64_t T = N / 16, G = K / kGroup;
-    if (M < 1 || T == 0 || G == 0) return;
-    const bool wide = T > (M == 1 && bits == 3 ? 16 : 8) * (int64_t)sms;
-    const bool big = G >= 32 && 2 * T > 3 * (int64_t)sms;
-    if (!(M >= 5 || wide || (big && (M >= 2 || bits == 4)) ||
-          (M >= 3 && (G >= 64 || (M == 4 && bits == 4 && T >= 4 * (int64_t)sms)))))
-        return;
+    if (M < 1 || T == 0 || G == 0 || !batch_takes(M, G, T, bits, sms)) return;
     const int nb = M > 8 ? 2 : 1;
     double best = 1e300;
     for (int tw = 1; tw <= 2; ++tw)
@@ -353,8 +369,9 @@ void plan_batch(int64_t M, int64_t K, int64_t N, int bits, int sms, laq_gemm_con
                 const double loop = (double)((gc + wk - 1) / wk) *
                                     (320.0 + tw * (300.0 + 290.0 * (nb - 1)));
                 const int64_t waves = fit2 > 0 ? (ctas + fit2 - 1) / fit2 : ctas;
+                const double pair = cl >= 7 && gc <= (T <= sms ? 3 : 2) ? 1.3 : 1.05;  // two per SM
                 const double cost = ctas <= fit1 ? fixed + loop
-                                                 : (double)waves * (1.05 * fixed + 1.5 * loop);
+                                                 : (double)waves * (pair * fixed + 1.5 * loop);
                 if (cost < best) {
                     best = cost;
                     out->reserved[0] = kBatchTag;

@@ -169,3 +169,25 @@ def test_plan_names_a_valid_batch_shape(bits, M):
                                       c.reserved[1] >> 16)
                 assert c.reserved[0] == TAG and tw in (1, 2) and slots in (1, 2, 4, 8)
                 assert 1 <= cluster <= min(8, K // 128)
+
+
+@pytest.mark.parametrize("M,K,N,bits,batch", [
+    # where chains of calls time the general kernel the faster one, by up to a third ...
+    (4, 512, 12288, 4, False), (4, 1024, 12288, 4, False), (4, 2048, 12288, 4, False),
+    (2, 256, 32768, 3, False), (2, 1024, 24576, 4, False), (1, 512, 24576, 4, False),
+    (1, 4096, 6144, 4, False), (1, 2560, 40960, 3, False), (3, 8192, 1024, 3, False),
+    (4, 9728, 512, 4, False), (3, 9728, 2560, 3, False),
+    # ... and where the batch kernel is
+    (4, 2560, 19456, 4, True), (4, 9728, 2560, 3, True), (3, 9728, 2560, 4, True),
+    (2, 4096, 24576, 3, True), (1, 4096, 24576, 4, True), (1, 12288, 4096, 4, True),
+    (3, 256, 32768, 3, True), (1, 2560, 151936, 3, True), (5, 128, 16, 3, True)])
+def test_plan_takes_the_faster_kernel(M, K, N, bits, batch):
+    assert (laq.laq_gemm_plan(M, K, N, bits, 152).batch is not None) == batch
+
+
+@pytest.mark.parametrize("M,K,N", [(8, 2048, 1152), (16, 2048, 1152), (8, 3072, 1152), (8, 2048, 1024)])
+def test_plan_does_not_fill_the_device_with_short_clusters(M, K, N):
+    """Two CTAs per SM of 2 or 3 groups each in clusters of 8 (4.3 us a call at 2048 x 1152 W4 M = 8):
+    slower than the general kernel (3.35) and than half the CTAs (3.0)."""
+    tw, slots, cluster = laq.laq_gemm_plan(M, K, N, 4, 152).batch
+    assert cluster < 7 or -(-(N // 16) // (tw * slots)) * cluster <= 152
