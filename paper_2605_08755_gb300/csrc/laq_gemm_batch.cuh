@@ -339,7 +339,6 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
         for (int i = 0; i < nw; ++i) {
             issue(i + S - 1 < nw, ring_s + prev);
             uint32_t B[NB][8][2];
-            float4 sp[NB];  // (S, P) of batch rows 8h + 2c and 8h + 2c + 1
 #pragma unroll
             for (int h = 0; h < NB; ++h) {
 #pragma unroll
@@ -350,7 +349,6 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
                     B[h][2 * q + 1][0] = v.z;
                     B[h][2 * q + 1][1] = v.w;
                 }
-                sp[h] = spp[h * 4];
             }
             cp_async_wait(S - 1);
             const uint8_t* rec = ring_w + cur;
@@ -368,12 +366,6 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
                         *reinterpret_cast<const uint2*>(rec + t * F::kBytes + 512 + lane * 8);
                     wd[4] = c1.x; wd[5] = c1.y;
                 }
-                float2 szv[2];  // columns R and R + 8 of the tile
-#pragma unroll
-                for (int r = 0; r < 2; ++r) {
-                    const uint32_t w = szp[16 * t + 8 * r];
-                    szv[r] = __half22float2(*reinterpret_cast<const __half2*>(&w));
-                }
                 float D[2][NB][4];
 #pragma unroll
                 for (int e = 0; e < 2; ++e)
@@ -389,15 +381,23 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
                     for (int h = 0; h < NB; ++h)
                         mma16816(D[j & 1][h], a[j][0], a[j][1], a[j][2], a[j][3], B[h][j][0],
                                  B[h][j][1]);
+                float2 szv[2];  // columns R and R + 8 of the tile
 #pragma unroll
-                for (int h = 0; h < NB; ++h)
+                for (int r = 0; r < 2; ++r) {
+                    const uint32_t w = szp[16 * t + 8 * r];
+                    szv[r] = __half22float2(*reinterpret_cast<const __half2*>(&w));
+                }
+#pragma unroll
+                for (int h = 0; h < NB; ++h) {
+                    const float4 sp = spp[h * 4];  // (S, P) of batch rows 8h + 2c and 8h + 2c + 1
 #pragma unroll
                     for (int v = 0; v < 4; ++v) {  // y += s (D - P - z S)
-                        const float S_ = v & 1 ? sp[h].z : sp[h].x, P_ = v & 1 ? sp[h].w : sp[h].y;
-                        const float d = D[0][h][v] + D[1][h][v] - P_;
-                        yacc[t][h][v] =
-                            fmaf(szv[v >> 1].x, fmaf(-szv[v >> 1].y, S_, d), yacc[t][h][v]);
+                        const float d = D[0][h][v] + D[1][h][v] - (v & 1 ? sp.w : sp.y);
+                        yacc[t][h][v] = fmaf(szv[v >> 1].x,
+                                             fmaf(-szv[v >> 1].y, v & 1 ? sp.z : sp.x, d),
+                                             yacc[t][h][v]);
                     }
+                }
             }
 #pragma unroll
             for (int q = 0; q < 4; ++q) xq[q] += Wk * NB * 128;
