@@ -7,7 +7,6 @@ torch = pytest.importorskip("torch")
 
 import paper_2605_08755_gb300 as laq  # noqa: E402
 from oracle import c_oracle as co  # noqa: E402
-from oracle import decoder as dec  # noqa: E402
 from paper_2605_08755_gb300 import _lib, inputs  # noqa: E402
 
 TAG = 0x4c424154
@@ -34,9 +33,10 @@ def prepared(K, N, bits, seed):
 
 
 def check(Y, ref, X, q):
-    """One fp16 rounding, and fp32 sums: a group's accumulator is as large as sum |x_k| times the
+    """One fp16 rounding, and fp32 sums: a group's accumulators are as large as sum |x_k| times the
     largest extraction offset (1024) plus the largest code, rounded about 2^-24 of that per
-    addition over 8 MMAs and the start value (16 allowed), times the group's scale."""
+    addition over 8 MMAs, the sum of the two chains, P and z S (16 allowed), times the group's scale.
+    (A bound for gross errors at every shape; how exact the sums are is tested below.)"""
     codes, s, z = q
     G = s.shape[0]
     mag = np.abs(X.astype(np.float64)).reshape(X.shape[0], G, 128).sum(-1) * 1040
@@ -104,6 +104,21 @@ def test_phases_and_edges(bits, M, K, N, shape):
     check(Y.cpu().numpy(), co.gemm(X, *q), X, q)
 
 
+def check_prologue(Y, Z, xin):
+    """Y with the prologue against Z, the plain GEMM of the input rounded from 64 bits.  The
+    prologue's input is within 2^-20 of the exact one (fp32 sums and reciprocals), so it rounds apart
+    where that is within 2^-20 of a tie: K 2^-9 of the K elements expected, 8 more allowed, each by
+    one fp16 step (2^-10 of it) of either sign.  8 standard deviations of their sum through weights of
+    root mean square 0.02, one rounding of each output, and the plain kernel's sums in another order
+    where the two stage K in phases of other lengths."""
+    Y, Z = Y.cpu().numpy().astype(np.float64), Z.cpu().numpy().astype(np.float64)
+    K = xin.shape[1]
+    rms = np.sqrt(np.square(xin.astype(np.float64)).mean())
+    bound = (8 * np.sqrt(8 + K * 2.0 ** -9) * 2.0 ** -10 * rms * 0.02 + 2.0 ** -10 * np.abs(Z)
+             + 2.0 ** -12 * np.sqrt(np.square(Z).mean()))
+    assert np.isfinite(Y).all() and (np.abs(Y - Z) <= bound).all(), (np.abs(Y - Z) / bound).max()
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("M,K", [(1, 1408), (3, 1408), (7, 1408), (8, 256), (16, 1408),
                                  (16, 12288)])   # the last: several phases, two passes over X and R
@@ -113,21 +128,80 @@ def test_prologues(M, K):
     dev = lambda a: torch.from_numpy(a).cuda()
     x, r = inputs.activations(M, K, seed=2), inputs.activations(M, K, seed=3)
     w = inputs.norm_weight(K, seed=4)
-    xin, h = dec.rmsnorm(x, w, 1e-6, r)
+    h = (x.astype(np.float32) + r.astype(np.float32)).astype(np.float16)  # one fp16 sum: exact
+    h64 = h.astype(np.float64)
+    xin = (h64 / np.sqrt(np.square(h64).mean(-1, keepdims=True) + 1e-6) * w).astype(np.float16)
     gu = inputs.activations(M, 2 * K, seed=5)
+    g64 = gu.astype(np.float64)
+    act = (g64[:, :K] / (1 + np.exp(-g64[:, :K])) * g64[:, K:]).astype(np.float16)
     for shape in ((2, 4, 1), (1, 2, 3), (2, 8, 8)):
         cfg = batch_config(*shape)
         hd = torch.empty((M, K), dtype=torch.float16, device="cuda")
         Y = _lib.laq_gemm_wxg128_prologue(dev(x), packed, s, z, bits, _lib.PROLOGUE_RMSNORM,
                                           R=dev(r), R_out=hd, w=dev(w), eps=1e-6, config=cfg)
-        Z = _lib.laq_gemm_wxg128_prologue(dev(gu), packed, s, z, bits, _lib.PROLOGUE_SILU_MUL,
+        check_prologue(Y, laq.laq_gemm_wxg128(dev(xin), packed, s, z, bits, config=cfg), xin)
+        assert np.array_equal(hd.cpu().numpy(), h)
+        Y = _lib.laq_gemm_wxg128_prologue(dev(gu), packed, s, z, bits, _lib.PROLOGUE_SILU_MUL,
                                           config=cfg)
+        check_prologue(Y, laq.laq_gemm_wxg128(dev(act), packed, s, z, bits, config=cfg), act)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape", [(2, 4, 1), (1, 2, 3), (2, 8, 8)])
+@pytest.mark.parametrize("kind", ["plain", "norm", "silu"])
+def test_non_finite_rows_stay_in_their_rows(shape, kind):
+    bits, M, K, N = 4, 8, 1408, 336
+    q, packed, s, z = prepared(K, N, bits, seed=1)
+    w = torch.from_numpy(inputs.norm_weight(K, seed=4)).cuda()
+    x = torch.from_numpy(inputs.activations(M, K * (2 if kind == "silu" else 1), seed=2)).cuda()
+    r = torch.from_numpy(inputs.activations(M, K, seed=3)).cuda()
+
+    def run(x):
+        if kind == "plain":
+            return laq.laq_gemm_wxg128(x, packed, s, z, bits, config=batch_config(*shape))
+        if kind == "silu":
+            return _lib.laq_gemm_wxg128_prologue(x, packed, s, z, bits, _lib.PROLOGUE_SILU_MUL,
+                                                 config=batch_config(*shape))
+        return _lib.laq_gemm_wxg128_prologue(x, packed, s, z, bits, _lib.PROLOGUE_RMSNORM, R=r, w=w,
+                                             eps=1e-6, config=batch_config(*shape))
+    clean, bad = run(x), x.clone()
+    bad[1, 5], bad[4, K - 1], bad[6, 700] = float("inf"), float("nan"), -float("inf")
+    Y = run(bad)
+    keep = [0, 2, 3, 5, 7]
+    assert torch.equal(Y[keep], clean[keep])
+    assert not torch.isfinite(Y[4]).any()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape", [(2, 8, 1), (2, 4, 3), (1, 2, 8)])
+@pytest.mark.parametrize("M", [3, 16])
+def test_dependent_launches_wait(shape, M):
+    """Layers of plain, norm and SiLU calls, each reading what the one before it writes (X, R, gate|up),
+    overlapped by programmatic dependent launch and not: the same bits."""
+    bits, H, I, layers = 3, 1408, 1024, 12
+    o, gu, dn = (prepared(K, N, bits, seed=K + N)[1:] for K, N in ((H, H), (H, 2 * I), (I, H)))
+    w = torch.from_numpy(inputs.norm_weight(H, seed=4)).cuda()
+    x0 = torch.from_numpy(inputs.activations(M, H, seed=2)).cuda()
+    f16 = dict(dtype=torch.float16, device="cuda")
+
+    def run(pdl):
+        cfg = batch_config(*shape, pdl)
+        res = [torch.zeros((M, H), **f16), torch.empty((M, H), **f16)]
+        x, a = x0.clone(), torch.empty((M, H), **f16)
+        g, out = torch.empty((M, 2 * I), **f16), []
         torch.cuda.synchronize()
-        for y, ref in ((Y, co.gemm(xin, *q)), (Z, co.gemm(dec.silu_mul(gu), *q))):
-            err = np.abs(y.cpu().numpy().astype(np.float64) - ref).max()
-            assert err <= 5e-3 * np.abs(ref).max() + 1e-3  # the GEMV tolerance: inputs round apart
-        assert np.allclose(hd.cpu().numpy().astype(np.float64), h.astype(np.float64), rtol=1e-3,
-                           atol=1e-7)
+        for layer in range(layers):
+            laq.laq_gemm_wxg128(x, *o, bits, Y=a, config=cfg)
+            _lib.laq_gemm_wxg128_prologue(a, *gu, bits, _lib.PROLOGUE_RMSNORM, Y=g,
+                                          R=res[layer % 2], R_out=res[1 - layer % 2], w=w, eps=1e-6,
+                                          config=cfg)
+            _lib.laq_gemm_wxg128_prologue(g, *dn, bits, _lib.PROLOGUE_SILU_MUL, Y=x, config=cfg)
+        torch.cuda.synchronize()
+        return x, res[0], res[1]
+    want = run(0)
+    assert all(torch.isfinite(t).all() and t.any() for t in want)
+    for _ in range(5):
+        assert all(torch.equal(p, q) for p, q in zip(run(1), want))
 
 
 @pytest.mark.gpu
