@@ -218,12 +218,16 @@ __global__ void __launch_bounds__(128) qk_norm_rope_kernel(
 // (m16n8k16, fp16 operands, fp32 accumulation):
 //   scores^T = K q^T: A the 16 tokens' K rows straight from ldmatrix, B the q heads (fp16, as
 //     stored; the products are exact);
-//   out^T += V^T P^T: A from ldmatrix.trans, B the probabilities after a movmatrix transpose.
-//     They stay at fp32 precision: P = hi + lo with both halves fp16.  For G <= 4 the MMA's 8
-//     columns are 4 heads' hi and 4 heads' lo (q's B columns 4-7 repeat heads 0-3, so the lanes
-//     that would idle hold the same probabilities and contribute their low halves); WIDE
-//     (G = 5..8) issues one MMA for each half.  hi + lo is P to ~2^-22; p is scaled by 2^15 (it
-//     cancels against the sum of p), so that its small values stay above fp16's range.
+//   out^T += V^T P^T: A from ldmatrix.trans, B the probabilities after a movmatrix transpose, as
+//     P = hi + lo with both halves fp16: 22 to 23 significand bits of P's 24, so within one fp32 unit
+//     in the last place of p (p is scaled by 2^15, which cancels against the sum of p, so that its small
+//     values stay above fp16's range).  For G <= 4 the MMA's 8 columns are 4 heads' hi and 4 heads' lo
+//     (q's B columns 4-7 repeat heads 0-3, so the lanes that would idle hold the same probabilities and
+//     contribute their low halves); WIDE (G = 5..8) issues one MMA for each half.
+// The tensor core truncates what it adds, so no sum grows inside it: the 8 MMAs of a score and the
+// steps of out^T start from zero and are added in fp32.  (Kept in one accumulator, a warp's 32 steps
+// of a row of 8192 tokens left 0.29 % of the outputs rounded apart from 64 bits where V has mean 1, 0.005
+// % here and with fp32 FMAs throughout; the fp16 rounding is 2.08e-4 of the result in either.)
 // The warps' results meet in shared memory, the CTAs' through distributed shared memory: CTA r of
 // the cluster combines the head dimensions [128 r / C, 128 (r + 1) / C) in rank order and stores
 // fp16, so a call needs one launch and no scratch.  (Partials in a workspace and a combine kernel,
@@ -455,21 +459,26 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 2) attn_kernel(const AttnPara
             *reinterpret_cast<uint2*>(p.v_cache + off) = vnew;
             __syncwarp();
         }
-        // scores: sc[v] is token r + 8 (v / 2), column 2c + v % 2 (two chains)
-        float sc[4] = {0.f, 0.f, 0.f, 0.f}, sd[4] = {0.f, 0.f, 0.f, 0.f};
+        // scores: sc[v] is token r + 8 (v / 2), column 2c + v % 2
+        float sc[4], se[8][4];
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks) {
             uint32_t a[4];
             ldsm4(kb + (krow ^ (ks << 5)), a);  // chunks 2 ks and 2 ks + 1 of the 16 tokens
-            mma16816(ks & 1 ? sd : sc, a[0], a[1], a[2], a[3], qb[ks][0], qb[ks][1]);
+            se[ks][0] = se[ks][1] = se[ks][2] = se[ks][3] = 0.f;
+            mma16816(se[ks], a[0], a[1], a[2], a[3], qb[ks][0], qb[ks][1]);
         }
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+            sc[v] = ((se[0][v] + se[1][v]) + (se[2][v] + se[3][v])) +
+                    ((se[4][v] + se[5][v]) + (se[6][v] + se[7][v]));
         const int left = n - s * kStep;  // (>= 16 in all but the last step)
         float nm[2];
         bool grew = false;
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-            sc[e] = r < left ? sc[e] + sd[e] : -INFINITY;
-            sc[2 + e] = r + 8 < left ? sc[2 + e] + sd[2 + e] : -INFINITY;
+            sc[e] = r < left ? sc[e] : -INFINITY;
+            sc[2 + e] = r + 8 < left ? sc[2 + e] : -INFINITY;
             float v = fmaxf(sc[e], sc[2 + e]);
             v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 4));
             v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 8));
@@ -516,7 +525,10 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 2) attn_kernel(const AttnPara
         for (int t = 0; t < 8; ++t) {
             uint32_t a[4];  // V^T: dimensions 16 t .. 16 t + 15 of the 16 tokens
             ldsm4t(vb + vrow + (((2 * t + vj) ^ (lane & 7)) << 4), a);
-            mma16816(acc[t], a[0], a[1], a[2], a[3], bh[0], bh[1]);
+            float d[4] = {0.f, 0.f, 0.f, 0.f};
+            mma16816(d, a[0], a[1], a[2], a[3], bh[0], bh[1]);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) acc[t][v] += d[v];
             if (WIDE) mma16816(acl[WIDE ? t : 0], a[0], a[1], a[2], a[3], bl[0], bl[1]);
         }
         __syncwarp();  // every lane is done with the slot

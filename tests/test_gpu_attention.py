@@ -103,3 +103,21 @@ def test_attention_non_finite_values():
     kc[~np.isfinite(kc)] = 0
     ref = dec.attention(q, kc, vc, [150], SCALE).astype(np.float64)
     check(np.where(bad, 0, out[0]), np.where(bad, 0, ref[0]))
+
+
+@pytest.mark.parametrize("G,M", [(4, 320), (8, 320)])
+def test_sums_over_many_steps_stay_exact(G, M):
+    """One CTA per row, so a warp adds up 16 steps: of values with mean 1 and nearly equal weights
+    every sum grows to the end.  A relative error r rounds about 1500 r of the fp16 outputs apart from
+    64 bits (an fp16 step is 2^-10 to 2^-11 of its value); fp32 sums stay within 2^-22 of the result:
+    3.6e-4 of them.  (Sums kept inside the tensor core, which truncates: 1e-3 and more.)"""
+    L, Hkv = 2048, 1
+    g = torch.Generator(device="cuda").manual_seed(G)
+    f16 = lambda *shape: torch.randn(shape, generator=g, device="cuda").half()
+    q, kc, vc = f16(M, G * Hkv, D), f16(M, Hkv, L, D), (f16(M, Hkv, L, D).float() + 1).half()
+    lens = torch.full((M,), L, dtype=torch.int32, device="cuda")
+    out = _lib.laq_attention_decode(q, kc, vc, lens, SCALE,
+                                    _lib.attention_workspace(M, G * Hkv, L, "cuda"))
+    ref = torch.cat([torch.softmax(q[m:m + 1].double() @ kc[m].double().mT * SCALE, -1)
+                     @ vc[m].double() for m in range(M)])
+    assert (out != ref.half()).double().mean() <= 3.6e-4
