@@ -11,7 +11,7 @@ first replay's kernels follow the eager run's: for a graph form with L launches 
 ``-k regex:gemm_kernel -s L -c 4`` selects one launch of each projection of the replay's first
 layer; for a chain form ``-k regex:chain_kernel -s 1 -c 1`` and for a planned form
 ``-k regex:pass_kernel -s 1 -c 1`` select the replay's single launch.
-""""""
+"""
 import argparse
 import json
 

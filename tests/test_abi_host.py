@@ -28,6 +28,14 @@ def declared_functions():
     return sorted(set(re.findall(r"\b(laq_[a-z0-9_]+)\s*\(", text)))
 
 
+def test_every_program_of_the_package_parses():
+    for folder, _, files in os.walk(os.path.dirname(_lib.__file__)):
+        for name in files:
+            if name.endswith(".py"):
+                path = os.path.join(folder, name)
+                compile(open(path).read(), path, "exec")
+
+
 def test_header_declares_the_abi():
     names = declared_functions()
     assert set(names) == set(_lib.EXPORTS)
