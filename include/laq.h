@@ -410,8 +410,9 @@ size_t laq_attention_workspace_bytes(int64_t M, int32_t Hq, int64_t L_max);
  * n = len[m] (device) clamped to [0, L_max]; a row with n = 0 gets zeros.  q, out [M][Hq][D],
  * caches [M][Hkv][L_max][D], D = 128, Hq / Hkv <= 8.  One launch (a cluster of CTAs per row and
  * kv head), or, for long caches of few rows and kv heads, partials in `workspace` (max, sum of
- * exponentials, weighted V sum) and a second launch that combines them; summation orders are
- * fixed (deterministic).  Before the preceding kernel has finished, the kernel only reads len and
+ * exponentials, weighted V sum) and a second launch that combines them.  Summation orders are
+ * fixed for given M, Hkv and L_max (deterministic), but how a row's tokens are split follows from
+ * these, so the same row can round differently in another batch or with another cache capacity.  Before the preceding kernel has finished, the kernel only reads len and
  * prefetches cache rows into L2; everything its results depend on is read afterwards.
  * workspace_bytes >= laq_attention_workspace_bytes(M, Hq, L_max)
  * (LAQ_ERR_WORKSPACE otherwise; 4-byte aligned).  Both caches 16-byte aligned.

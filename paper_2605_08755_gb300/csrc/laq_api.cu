@@ -102,7 +102,9 @@ laq_status check_config(const laq_gemm_config* c) {
 
 int ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 
-// Launch-shape plan: tiles per CTA (NT), K split over a cluster (C), warps and ring depth.
+// Launch-shape plan of the general kernel: tiles per CTA (NT), K split over a cluster (C), warps and
+// ring depth.  Where batch_takes() the shape (M >= 5 always) the batch kernel runs instead, and the
+// rules for it below serve a plan whose fields were changed or that was made without the batch shape.
 //  * M = 1, 2: the cheapest split by estimated SM time -- records per warp plus a start cost of
 //    two records' time per wave of CTAs, x the waves (two 8-warp CTAs per SM at a time), x 1.3
 //    when two CTAs share an SM (16 warps retire a record in ~0.65x the time of 8; measured on
@@ -295,25 +297,25 @@ BatchShape decode_batch(const laq_gemm_config& c, int64_t M) {
 }
 
 // Whether the batch kernel takes a shape (t = tiles per SM), as timed on GB300 by
-// measure/kernel_choice.py, us: chains of dependent calls of one size (ratio general / batch kernel
-// in their planned shapes) and whole decoder layers.
-//  * M = 5..16: always.  Chains 0.97 to 2.9 (M = 5..8, 512 or 1024 columns and 28 groups or more 0.90 to
-//    0.98, calls of 3.4 to 3.8 us); Qwen3-4B W3 M = 8 31.8 -> 26.1 us per layer, M = 16 48.4 -> 34.5,
-//    Qwen3-8B W3 M = 8 64.1 -> 36.9, M = 16 85.3 -> 48.8, a 1408-wide decoder W4 M = 8 16.6 -> 15.5.
-//  * M = 3, 4, t > 8: always (1.0 to 2.2).  M = 2, t > 8: K of 16 groups (W4: 11) or more, 0.99 to
-//    1.6; below, 0.74 to 1.1.  M = 1, t > 8, W4: 18 groups or more, 1.02 to 1.5; below, 0.72 to
-//    1.5.  M = 1, W3: t > 24 and 16 groups or more, 1.06 to 1.38 (2560 x 151936 52.1 -> 38.7 us); up to
-//    t = 24, 0.72 to 1.3, and the Qwen3-8B gate|up (t = 10) 33.9 us per layer here, 32.5 there.
-//  * K of 32 groups or more, t > 1.5, M = 2..4: 0.90 to 2.0 in chains (9728 columns at M = 2, W3 0.84);
-//    the sizes below 1 (t <= 4 and K under 40 groups) gain where their neighbours run this kernel too:
-//    Qwen3-8B M = 2 39.4 -> 34.6 us per layer (W4 43.2 -> 34.2), 35.4 with the general kernel for its
-//    4096 x 4096.  M = 1, W4: t > 4 or K of 64 groups, 0.95 to 1.6 (Qwen3-8B 35.9 -> 33.9); below 0.77
-//    to 0.95.
-//  * K of 72 groups or more, M = 3, 4, narrower outputs: t >= 1.25 from 64 groups 1.34 to 1.6; t >=
-//    0.5 from 88 groups 1.03 to 1.33; t >= 1 from 72 groups at M = 4 and W4 M = 3, 1.02 to 1.1
-//    (Qwen3-4B M = 4 24.1 -> 23.8 us per layer); below 0.88 to 1.0.
-//  * M = 4, W4, t > 4, K of 20 groups or more: 1.1 to 1.8 (Qwen3-4B with its gate|up here 24.05 us per
-//    layer, 24.6 without); shorter K 0.65 to 1.0.
+// measure/kernel_choice.py: ratios (general / batch kernel, each in its planned shape) in chains of
+// dependent calls of one size, us per whole decoder layer with every projection on the general kernel ->
+// as planned.
+//  * M = 5..16: always.  Ratios 0.94 (5 % below 1.04) to 3.0; M = 5..8, 512 or 1024 columns, 28 groups or
+//    more 0.90 to 1.6 (calls of 3.4 to 3.9 us).  Qwen3-4B W3 M = 8 31.9 -> 25.7, M = 16 48.3 -> 33.7;
+//    Qwen3-8B W3 M = 8 64.6 -> 36.1, M = 16 85.6 -> 48.2; a 1408-wide decoder W4 M = 8 16.6 -> 15.4.
+//  * t > 8.  M = 3, 4: always, 1.0 to 2.2.  M = 2: K of 16 groups (W4: 11) or more, 1.01 to 2.1; below
+//    0.75 to 1.6.  M = 1, W4: 18 groups or more, 0.96 (5 % below 1.03) to 1.66; below 0.72 to 1.5.
+//    M = 1, W3: t > 24 and 16 groups or more, 1.02 to 1.39 (2560 x 151936 51.2 -> 37.9 us); up to t = 24
+//    0.72 to 1.5, and an 8192-wide decoder's gate|up (t = 23.6) 118.2 -> 121.4 us per layer.
+//  * K of 32 groups or more, t > 1.5.  M = 2..4: 0.95 (5 % below 1.07) to 2.3; t <= 4 and K under 40
+//    groups 0.86 to 1.5, but those gain where their neighbours run this kernel too: Qwen3-8B M = 2
+//    39.6 -> 34.1 (W4 43.3 -> 33.9), with the general kernel for its 4096 x 4096 34.8 (34.7).  M = 1, W4:
+//    t > 4 or 64 groups, 0.96 to 1.66 (Qwen3-8B 36.0 -> 33.6); below 0.82 to 1.1.
+//  * Narrower outputs, M = 3, 4.  t >= 1.25 from 64 groups 1.36 to 1.64; t >= 0.5 from 88 groups 1.0 to
+//    1.6; t >= 1 from 72 groups at M = 4 and W4 M = 3 1.03 to 1.09 (Qwen3-4B M = 4 24.1 -> 23.8); the rest
+//    of 64 groups or more 0.89 to 1.05.
+//  * M = 4, W4, t > 4, 20 groups or more: 1.13 to 1.5 (Qwen3-4B 23.9, without its gate|up 24.5); shorter
+//    K 0.66 to 1.09.
 bool batch_takes(int64_t M, int64_t G, int64_t T, int bits, int64_t sms) {
     if (M >= 5) return true;
     const bool w4 = bits == 4;

@@ -231,8 +231,8 @@ __global__ void __launch_bounds__(128) qk_norm_rope_kernel(
 // The warps' results meet in shared memory, the CTAs' through distributed shared memory: CTA r of
 // the cluster combines the head dimensions [128 r / C, 128 (r + 1) / C) in rank order and stores
 // fp16, so a call needs one launch and no scratch.  (Partials in a workspace and a combine kernel,
-// fp32 FMAs and a 4-shuffle score: 13.3 us a call for one row of 2048 tokens, 138 us for 16 rows of
-// 2048 .. 8192; this form 6.7 and 59 us, 5.7 TB/s.)  Where the clusters of all (row, kv head)
+// fp32 FMAs and a 4-shuffle score: 13.3 us a call for one row of 2048 tokens, 129 us for 16 rows of
+// 2048 .. 8192; this form 6.7 and 62 us, 5.4 TB/s.)  Where the clusters of all (row, kv head)
 // pairs leave most SMs idle and the rows may be long, S clusters share a pair, write fp32 partials
 // (acc[D], max, sum) to the workspace, and attn_combine_kernel adds them in order.
 // Bound: HBM for long batches; for one short row the latency of a dependent launch (4.6 us at 256

@@ -1,5 +1,5 @@
 // laq_gemm_batch.cuh -- the dequantize-fused GEMM kernel for batches (M = 5..16, and M = 1..4 on
-// wide outputs; the lines stand at plan_batch in laq_api.cu), included by the translation units
+// wide outputs; the lines stand at batch_takes in laq_api.cu), included by the translation units
 // that instantiate it (laq_gemm_batch.cu: plain X, laq_gemm_prologue.cu: X made by a fused prologue).
 // Same records, extraction and group algebra as laq_gemm_kernel.cuh:
 // D = sum_k (c_k + q_k) x_k on the tensor cores, y += s (D - P - z S) per group, with
@@ -27,11 +27,13 @@
 // 8 warps per CTA, two CTAs per SM: Wt tile slots x Wk = 8 / Wt teams that split the CTA's
 // groups, K split further over a cluster of 1..8 CTAs (any size, so that the grid fills the SMs),
 // reduced through distributed shared memory in rank order.
-// Measured, us per call in a chain of calls: 4096 x 24576 W3 M = 16 gemm_kernel 42.9, this one 19.9;
-// 2560 x 19456 W3 M = 8 10.8, 9.1; 9728 x 2560 W4 M = 4 6.7, 6.4.  Of the first, the group loop takes
-// 8.6 in the median CTA, the rest is launch, 45 KB of X per CTA, S and P, reduction.  Its first
-// version took 31.2 (S and P with conversions and branches, integer divisions in the reduction),
-// 20.9 without those, and the rest of the way came with plain loads of X.
+// Measured, us per call in a chain of calls (measure/kernel_choice.py --chain): 4096 x 24576 W3 M = 16
+// gemm_kernel 42.3, this one 19.9; 2560 x 19456 W3 M = 8 10.8, 9.1, W4 M = 4 9.3, 8.0; 9728 x 2560 W4
+// M = 4 6.7, 6.3; 2560 x 151936 W3 M = 1 51.2, 37.9.  Of the first about half is outside the group
+// loop: launch, 45 KB of X per CTA, S and P, reduction.  S and P with conversions and branches and
+// integer divisions in the reduction cost 10 us of it, cp.async for X 1.  The scales, zeros and group
+// sums are loaded after the products, not held across them: at NB = TW = 2 the second accumulator
+// chain otherwise spills (16 Qwen3-8B layers at M = 16 782 us, 766 so).
 #pragma once
 #include "laq_gemm_kernel.cuh"
 
@@ -111,7 +113,7 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2) gemm_batch_kernel(const B
     // read once, h = fp16(X + R) is staged, its sums of squares come from the staged fragments and,
     // over a cluster, from its CTAs, and the staged rows are normalised in place.  (Reading all of X
     // and R in every CTA for the sums and the slice again for staging: 120 KB per CTA at M = 8, K =
-    // 2560, 4.2 us more per call than a plain GEMM; in place about 3.)
+    // 2560, 4.2 us more per call than a plain GEMM; in place 3.2.)
     const bool in_place = PRO && p.pro == kProRmsNorm && p.gc <= GP && C <= p.G;
     uint4* wsm = reinterpret_cast<uint4*>(inv_rms + 16 + 2 * 8 * 16);  // w of the slice
     bool first = true;

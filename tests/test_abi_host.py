@@ -236,6 +236,8 @@ def test_chain_static_argument_validation(L):
 
 
 def test_plan_shares_x_across_tiles_above_m_two(L):
+    """The general kernel's shapes, the faster ones among its own on GB300; where the plan names the
+    batch kernel too (M >= 5 always), they run once the plan is edited."""
     one = lambda K, N, bits: laq.laq_gemm_plan(1, K, N, bits, 152).as_dict()
     shape = lambda c: (c.tiles_per_cta, c.warps, c.cluster, c.stages)
     for bits in (3, 4):
